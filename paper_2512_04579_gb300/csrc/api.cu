@@ -75,6 +75,11 @@ struct gnmppi_s {
   std::vector<int> order;  // k_solve instance order
   int* d_order = nullptr;
   int solve_smem = 0;
+  // cluster Cholesky (0: none): CTAs per instance, shared memory, row plans
+  int cl_size = 0, cl_smem = 0;
+  double* d_Hs = nullptr;
+  int* d_cl_plan = nullptr;
+  int64_t* d_o_cl = nullptr;
   bool use_tc = false;
   // concurrency of the rollout groups and the solve CTA shape
   TuneCfg tune{};
@@ -101,6 +106,17 @@ struct gnmppi_s {
   std::vector<void*> allocs;
   std::string err;
 };
+
+// Opt kernel k into at least `smem` bytes of dynamic shared memory.  The
+// attribute belongs to the function, not to a handle, so it is only ever
+// raised: another handle may have opted in to more.
+template <typename K>
+static cudaError_t raise_smem(K k, int smem) {
+  cudaFuncAttributes at{};
+  cudaError_t e = cudaFuncGetAttributes(&at, k);
+  if (e != cudaSuccess || at.maxDynamicSharedSizeBytes >= smem) return e;
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+}
 
 static thread_local std::string g_create_err;  // errors raised before a handle exists
 
@@ -277,6 +293,7 @@ extern "C" int64_t gnmppi_check_count(void) {
 #endif
 }
 
+static gnmppi_status choose_cluster(gnmppi_t h, int optin, int nsm);
 static gnmppi_status build(gnmppi_t h, const gnmppi_instance_shape* shapes) {
   const gnmppi_problem& p = h->p;
   const int prec = p.precision;
@@ -526,6 +543,13 @@ static gnmppi_status build(gnmppi_t h, const gnmppi_instance_shape* shapes) {
       CK(cudaFuncSetAttribute(k_solve<float, 128>, cudaFuncAttributePreferredSharedMemoryCarveout, pct4));
     }
   }
+  {
+    int dev = 0, optin = 0, nsm = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    if ((st = choose_cluster(h, optin, nsm)) != GNMPPI_OK) return st;
+  }
   // default launch configuration (the autotuner may replace it): a batch no
   // larger than the SM count gets one SM per instance, and then 16 warps per
   // Cholesky shorten its serial steps; larger batches pair instances per SM
@@ -646,7 +670,108 @@ static SolveArgs solve_args(gnmppi_t h, int shrink) {
   a.Cl = h->d_Cl;
   a.shrink = shrink;
   a.order = h->d_order;
+  a.Hs = h->d_Hs;
+  a.cl_plan = h->d_cl_plan;
+  a.o_cl = h->d_o_cl;
   return a;
+}
+
+// ------------------------------------------------------ cluster Cholesky
+static cudaLaunchConfig_t cluster_config(int cs, int batch, int smem, cudaStream_t s, cudaLaunchAttribute* attr) {
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = (unsigned)cs;
+  attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(batch * cs));
+  cfg.blockDim = dim3(kClThreads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// Clusters of cs CTAs that the device holds at once (0: none, or the attributes are refused).
+template <typename TA>
+static int cluster_capacity(int cs, int smem) {
+  auto k = k_solve_cluster<TA>;
+  int n = 0;
+  cudaLaunchAttribute attr;
+  const cudaLaunchConfig_t cfg = cluster_config(cs, 1, smem, nullptr, &attr);
+  if (raise_smem(k, smem) != cudaSuccess ||
+      (cs > 8 && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+      cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
+template <typename TA>
+static cudaError_t cluster_launch(int cs, const SolveArgs& a, int batch, int smem, cudaStream_t s) {
+  cudaLaunchAttribute attr;
+  const cudaLaunchConfig_t cfg = cluster_config(cs, batch, smem, s, &attr);
+  return cudaLaunchKernelEx(&cfg, k_solve_cluster<TA>, a);
+}
+
+// CTAs per instance of the cluster Cholesky: of the sizes that leave every
+// instance its own SMs and fit shared memory, the smallest whose longest path
+// (cluster_path of the largest system) is within 2 % of the shortest, or the
+// next smaller ones if the device does not hold all those clusters at once;
+// none for systems of fewer than three panels, or when no size fits.
+// k_solve against this (n = 200): 768 -> 299 us at 1 instance (8 CTAs), 786 ->
+// 502 at 64 (2 CTAs); n = 400: 3809 -> 760 at 1 (14 CTAs), 3835 -> 1001 at 16
+// (6 CTAs); n = 50: 123 -> 82.
+static gnmppi_status choose_cluster(gnmppi_t h, int optin, int nsm) {
+  int nmax = 0;
+  for (auto& d : h->desc) nmax = std::max(nmax, d.n);
+  const int nblk = (nmax + CNB - 1) / CNB;
+  if (h->p.method != GNMPPI_METHOD_GN || nblk < 3 || nblk > kClMaxBlocks) return GNMPPI_OK;
+  std::vector<int> plan(nblk);
+  struct Size {
+    int cs, smem;
+    double path;
+  };
+  std::vector<Size> sizes;  // largest first
+  double best = 1e300;
+  for (int cs : {16, 14, 12, 10, 8, 7, 6, 5, 4, 3, 2}) {
+    if ((int64_t)cs * h->batch > nsm) continue;
+    const int64_t smem = 8 * (cl_fixed_doubles(nmax) + 256 * (int64_t)cluster_plan(nmax, cs, plan.data()));
+    if (smem + 2048 > optin) break;  // fewer ranks store more each
+    sizes.push_back({cs, (int)smem, (double)cluster_path(nmax, cs, plan.data())});
+    best = std::min(best, sizes.back().path);
+  }
+  size_t k = 0;
+  while (k + 1 < sizes.size() && sizes[k + 1].path <= 1.02 * best) ++k;
+  for (; k < sizes.size() && !h->cl_size; ++k) {
+    const int cap = h->p.precision == kFP64 ? cluster_capacity<double>(sizes[k].cs, sizes[k].smem)
+                                            : cluster_capacity<float>(sizes[k].cs, sizes[k].smem);
+    if (cap < h->batch) continue;
+    h->cl_size = sizes[k].cs;
+    h->cl_smem = sizes[k].smem;
+  }
+  if (!h->cl_size) return GNMPPI_OK;
+  std::vector<int> all;
+  std::vector<int64_t> off(h->batch);
+  std::map<int, std::vector<int>> by_n;
+  for (int b = 0; b < h->batch; ++b) {
+    const int n = h->desc[b].n;
+    std::vector<int>& q = by_n[n];
+    if (q.empty()) {
+      q.resize((n + CNB - 1) / CNB);
+      cluster_plan(n, h->cl_size, q.data());
+    }
+    off[b] = (int64_t)all.size();
+    all.insert(all.end(), q.begin(), q.end());
+  }
+  gnmppi_status st;
+  if ((st = dalloc(h, &h->d_Hs, 8 * h->n_nn)) != GNMPPI_OK) return st;
+  if ((st = dalloc(h, &h->d_cl_plan, sizeof(int) * all.size())) != GNMPPI_OK) return st;
+  if ((st = dalloc(h, &h->d_o_cl, sizeof(int64_t) * off.size())) != GNMPPI_OK) return st;
+  CK(cudaMemcpyAsync(h->d_cl_plan, all.data(), sizeof(int) * all.size(), cudaMemcpyHostToDevice, h->stream));
+  CK(cudaMemcpyAsync(h->d_o_cl, off.data(), sizeof(int64_t) * off.size(), cudaMemcpyHostToDevice, h->stream));
+  CK(cudaStreamSynchronize(h->stream));  // the host vectors are temporaries
+  return GNMPPI_OK;
 }
 
 // Assign the rollout groups to nb branches, heaviest first to the least
@@ -793,6 +918,7 @@ static gnmppi_status launch_iteration_t(gnmppi_t h, uint32_t it, int shrink, cud
   MARK(5);
   if (ON(5)) {
     if (!gn) k_mppi_step<<<h->batch, 256, 0, h->stream>>>(sa);
+    else if (h->tune.solve_nt == 512 && h->cl_size) CK(cluster_launch<TA>(h->cl_size, sa, h->batch, h->cl_smem, h->stream));
     else if (h->tune.solve_nt == 128) k_solve<TA, 128><<<h->batch, 128, h->solve_smem, h->stream>>>(sa);
     else if (h->tune.solve_nt == 512) k_solve<TA, 512><<<h->batch, 512, h->solve_smem, h->stream>>>(sa);
     else k_solve<TA, 256><<<h->batch, 256, h->solve_smem, h->stream>>>(sa);

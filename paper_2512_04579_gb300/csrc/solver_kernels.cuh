@@ -16,6 +16,7 @@
 #pragma once
 #include "common.cuh"
 #include "chol.cuh"
+#include "chol_cluster.cuh"
 
 namespace gnm {
 
@@ -44,6 +45,9 @@ struct SolveArgs {
   double* Cl;      // [kMaxL+1]
   int shrink;      // apply the covariance shrink after the update
   uint32_t it;     // iteration index (test injection)
+  double* Hs;              // cluster solve: the damped systems, both triangles, at InstDesc::o_nn
+  const int* cl_plan;      // cluster solve: block-row plans of the instances
+  const int64_t* o_cl;     // per-instance offsets into cl_plan
 };
 
 // p[0..count) = v (the default per-component sampling scale sigma0).
@@ -84,6 +88,17 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   __syncthreads();
   double t = 0.0;
   for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += red[i];
+  return t;
+}
+// block_sum for the first warp only (the last sum takes no FP64 slots of the others).
+__device__ __forceinline__ double block_sum_first(double v, double* red) {
+  v = warp_sum(v);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x < 32)
+    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += red[i];
   return t;
 }
 __device__ __forceinline__ double block_min(double v, double* red) {
@@ -386,6 +401,19 @@ __global__ void __launch_bounds__(256) k_gemm_nt(GemmArgs g) {
 // tau diag(A): the tensor-core Gram's entries carry ~1e-5 of sqrt(A_ii A_jj)
 // of rounding, and when K' is barely above n, S^2 is so small in some
 // directions that this rounding leaves A + lambda S^2 indefinite.
+__device__ __forceinline__ double system_entry(const double* __restrict__ A, const double* __restrict__ S2,
+                                               const double* __restrict__ s, bool lsq, double Keff, double lam,
+                                               double tau, int r, int c, int n) {
+  const int64_t i = (int64_t)r * n + c;
+  double t;
+  if (lsq) {
+    t = S2[i];
+  } else {
+    const double sc = Keff * s[r] * s[r];
+    t = (r == c) ? sc * sc : 0.0;
+  }
+  return A[i] + lam * t + ((r == c && lsq) ? tau * A[i] : 0.0);
+}
 __device__ __forceinline__ void build_system(const double* __restrict__ A, const double* __restrict__ S2,
                                              const double* __restrict__ s, bool lsq, double Keff, double lam,
                                              double tau, double* __restrict__ Hp, double* __restrict__ L, int n) {
@@ -396,15 +424,7 @@ __device__ __forceinline__ void build_system(const double* __restrict__ A, const
     while ((r + 1) * (r + 2) / 2 <= u) ++r;
     while (r * (r + 1) / 2 > u) --r;
     const int c = u - r * (r + 1) / 2;
-    const int64_t i = (int64_t)r * n + c;
-    double t;
-    if (lsq) {
-      t = S2[i];
-    } else {
-      const double sc = Keff * s[r] * s[r];
-      t = (r == c) ? sc * sc : 0.0;
-    }
-    const double h = A[i] + lam * t + ((r == c && lsq) ? tau * A[i] : 0.0);
+    const double h = system_entry(A, S2, s, lsq, Keff, lam, tau, r, c, n);
     Hp[u] = h;
     L[u] = h;
   }
@@ -581,6 +601,140 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_solve(SolveArgs a) {
     dsq += acc * acc;
   }
   dsq = block_sum(dsq, red);
+  if (tid == 0) {
+    st.chol_retries = retries;
+    st.lambda_used = lam;
+    st.step_norm = sqrt(dsq);
+    st.jac_mode_used = lsq ? 0 : 1;
+    if (I.lsq && !lsq) st.lsq_broken = 1;
+  }
+}
+
+// k_solve on a cluster of CTAs per instance (chol_cluster.cuh): every rank
+// factorises, substitutes and forms delta on its block rows; rank 0 also runs
+// the factorisation's serial chain and reports.
+template <typename TA>
+__global__ void __launch_bounds__(kClThreads, 1) k_solve_cluster(SolveArgs a) {
+  const int b = a.order[blockIdx.x / (unsigned)cl_size()];
+  InstState& st = a.st[b];
+  if (st.status != 0) return;  // uniform over the cluster: rank 0 writes it after a cluster barrier only
+  const InstDesc I = a.inst[b];
+  const int n = I.n, tid = threadIdx.x;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int fail, nrows;
+  __shared__ int rows[kClMaxBlocks];
+  __shared__ double red[32];
+  ClusterChol cc;
+  cc.size = cl_size();
+  cc.n = n;
+  cc.nblk = (n + CNB - 1) / CNB;
+  cc.rank = cl_my_rank();
+  cc.plan = a.cl_plan + a.o_cl[b];
+  cc.rows = rows;
+  cc.fail = &fail;
+  double* v = reinterpret_cast<double*>(smem_raw);
+  cc.m.ybuf = v;
+  cc.m.cbuf = v + 512;
+  cc.m.lbuf = v + 1536;
+  cc.m.col = v + 1792;
+  cc.m.pbuf = v + 1860;
+  cc.m.blk = cc.m.pbuf + (int64_t)cc.nblk * 256;
+  if (tid == 0) {
+    int c = 0;
+    for (int q = 0; q < cc.nblk; ++q)
+      if (cl_rank(cc.plan[q]) == cc.rank) rows[c++] = q;
+    nrows = c;
+  }
+  bool r0 = false;
+  for (int q = 0; q < cc.nblk; ++q) r0 = r0 || cl_rank(cc.plan[q]) == 0;
+  cc.rank0_rows = r0;
+  __syncthreads();
+  cc.nrows = nrows;
+
+  double* H = a.Hs + I.o_nn;
+  const double* A = a.A + I.o_nn;
+  const double* S2 = a.S2 + I.o_nn;
+  const double* s = a.s + I.o_U;
+  const double Keff = (double)(I.Kp - st.n_masked);
+  bool lsq = I.lsq != 0 && st.lsq_broken == 0;
+  double lam = a.cs.lambda;
+  int retries = 0;
+  bool ok = false;
+  const bool inj = a.cs.inj_kind != 0 && (int32_t)a.it == a.cs.inj_it;
+  for (int pass = 0; pass < 2 && !ok; ++pass) {  // the retry ladder of k_solve
+    if (pass == 1) {
+      if (!lsq) break;
+      lsq = false;
+      lam = a.cs.lambda;
+    }
+    const bool forced = inj && (a.cs.inj_kind == 2 || lsq);
+    for (retries = 0; retries <= 6; ++retries) {
+      double tau = 0.0;
+      retry_ladder<TA>(retries, lsq, a.cs.lambda, lam, tau);
+      const bool got = cc.factor(H, [&](int r, int c) { return system_entry(A, S2, s, lsq, Keff, lam, tau, r, c, n); });
+      if (got && !forced) {
+        ok = true;
+        break;
+      }
+    }
+  }
+  cl_arrive();  // H is complete, and the panel buffers may turn into vectors
+  cl_wait();
+  const ClVec w(cc.m.pbuf, n);
+  double gsq = 0.0;
+  for (int j = tid; j < n; j += blockDim.x) {
+    const double gj = a.g[I.o_U + j];
+    w.rhs[j] = -gj;
+    w.b[j] = -gj;
+    gsq += gj * gj;
+  }
+  if (cc.rank == 0) {
+    gsq = block_sum_first(gsq, red);
+    if (tid == 0) st.pr_norm = sqrt(gsq);  // |b|, b = P^T r
+  }
+  if (!ok) {
+    if (cc.rank == 0 && tid == 0) {
+      st.status = -3;
+      st.chol_retries = 7;
+      st.lambda_used = lam;
+    }
+    return;
+  }
+  cl_arrive();  // the vectors are set up before another rank writes to them
+  cl_wait();
+  // y = H^-1 rhs with iterative refinement, delta = S_used y, as in k_solve
+  cc.substitute(w, w.x);
+  for (int t = 0; t < a.cs.ir_steps; ++t) {
+    cc.residual(w, H);
+    __syncwarp();
+    cc.substitute(w, w.dx);
+    for (int j = tid; j < n; j += blockDim.x) w.x[j] += w.dx[j];
+    __syncthreads();
+  }
+  for (int j = tid; j < n; j += blockDim.x) {
+    const float h = (float)w.x[j];
+    w.yh[j] = h;
+    w.yl[j] = (float)(w.x[j] - (double)h);
+  }
+  __syncthreads();
+  const TA* P = reinterpret_cast<const TA*>(a.P) + I.o_P;
+  const int row = cc.my_row(), i = row * CNB + (tid & 15);
+  double acc = 0.0;
+  if (lsq) acc = cc.row_dot(w, P + I.sP, (int64_t)I.ldP);
+  if (row >= 0 && i < n) {
+    if (!lsq) acc = Keff * s[i] * s[i] * w.x[i];
+    if (GNM_IN(i, n)) {
+      a.delta[I.o_U + i] = acc;
+      a.y[I.o_U + i] = w.x[i];
+    }
+    cl_map(w.delta, 0)[i] = acc;
+  }
+  cl_arrive();
+  cl_wait();
+  if (cc.rank != 0) return;
+  double dsq = 0.0;
+  for (int j = tid; j < n; j += blockDim.x) dsq += w.delta[j] * w.delta[j];
+  dsq = block_sum_first(dsq, red);
   if (tid == 0) {
     st.chol_retries = retries;
     st.lambda_used = lam;
