@@ -68,8 +68,11 @@ struct gnmppi_s {
   uint32_t* d_W2 = nullptr;  // BF16 mode: W split into BF16 head and remainder (the contraction's B rows)
   int64_t n_x0 = 0, n_xref = 0, n_U = 0, n_dR = 0, n_W = 0, n_C = 0, n_P = 0, n_nn = 0, n_R = 0, n_RL = 0, n_L = 0;
   size_t szT = 8, szS = 8, szA = 8;
-  int4* d_tiles[3] = {nullptr, nullptr, nullptr};
-  int ntiles[3] = {0, 0, 0};
+  // FP64 products: row blocks (instance, block of 16 rows), all instances' and
+  // the LSQ ones', and the most columns of an instance's output
+  int2 *d_grows = nullptr, *d_grows_lsq = nullptr;
+  int ngrows = 0, ngrows_lsq = 0, nmax_u = 0;
+  int64_t nmax_R = 0;
   std::vector<Group> groups;
   int* d_all = nullptr;  // 0..batch-1
   std::vector<int> order;  // k_solve instance order
@@ -469,24 +472,26 @@ static gnmppi_status build(gnmppi_t h, const gnmppi_instance_shape* shapes) {
     CK(cudaMemcpyAsync(g.d_list, g.insts.data(), 4 * g.insts.size(), cudaMemcpyHostToDevice, h->stream));
     CK(cudaMemcpyAsync(g.d_bmap, g.bmap.data(), sizeof(int2) * g.bmap.size(), cudaMemcpyHostToDevice, h->stream));
   }
-  // GEMM tile maps (64 x 64 tiles)
-  std::vector<int4> tl[3];
-  for (int b = 0; b < h->batch; ++b) {
-    const InstDesc& d = h->desc[b];
-    const int tm = (d.n + 63) / 64;
-    for (int i = 0; i < tm; ++i) {
-      for (int j = 0; j < (d.nR + d.n + 63) / 64; ++j) tl[0].push_back(make_int4(b, i, j, 0));
-      for (int j = 0; j < tm; ++j) {
-        tl[1].push_back(make_int4(b, i, j, 0));
-        if (d.lsq) tl[2].push_back(make_int4(b, i, j, 0));
+  if (prec == kFP64) {
+    std::vector<int2> all_rows, lsq_rows;
+    for (int b = 0; b < h->batch; ++b) {
+      const InstDesc& d = h->desc[b];
+      h->nmax_u = std::max(h->nmax_u, d.n);
+      h->nmax_R = std::max<int64_t>(h->nmax_R, d.nR);
+      for (int i = 0; i < (d.n + 15) / 16; ++i) {
+        all_rows.push_back(make_int2(b, i));
+        if (d.lsq) lsq_rows.push_back(make_int2(b, i));
       }
     }
-  }
-  for (int k = 0; k < 3; ++k) {
-    h->ntiles[k] = (int)tl[k].size();
-    AL(h->d_tiles[k], sizeof(int4) * std::max<size_t>(1, tl[k].size()));
-    if (!tl[k].empty())
-      CK(cudaMemcpyAsync(h->d_tiles[k], tl[k].data(), sizeof(int4) * tl[k].size(), cudaMemcpyHostToDevice, h->stream));
+    h->ngrows = (int)all_rows.size();
+    h->ngrows_lsq = (int)lsq_rows.size();
+    AL(h->d_grows, sizeof(int2) * all_rows.size());
+    AL(h->d_grows_lsq, sizeof(int2) * lsq_rows.size());
+    CK(cudaMemcpyAsync(h->d_grows, all_rows.data(), sizeof(int2) * all_rows.size(), cudaMemcpyHostToDevice, h->stream));
+    if (!lsq_rows.empty())
+      CK(cudaMemcpyAsync(h->d_grows_lsq, lsq_rows.data(), sizeof(int2) * lsq_rows.size(), cudaMemcpyHostToDevice,
+                         h->stream));
+    CK(cudaStreamSynchronize(h->stream));  // the host vectors are temporaries
   }
 #undef AL
   // constants
@@ -832,6 +837,17 @@ constexpr int kNumPhases = 8;
 
 constexpr unsigned kAllPhases = (1u << kNumPhases) - 1;
 
+// One of the FP64 mode's products over every instance (S2: the LSQ ones).
+template <GemmKind KIND>
+static cudaError_t launch_gemm_f64(gnmppi_t h) {
+  const GemmArgs g{h->d_desc, h->d_st, KIND == kS2 ? h->d_grows_lsq : h->d_grows,
+                   (const double*)h->d_dR, (const double*)h->d_W, (double*)h->d_P, h->d_A, h->d_S2};
+  const int nrows = KIND == kS2 ? h->ngrows_lsq : h->ngrows;
+  const int64_t cols = (h->nmax_u + 15) / 16 + (KIND == kContract ? (h->nmax_R + 15) / 16 : 0);
+  k_gemm_f64<KIND><<<dim3((unsigned)nrows, (unsigned)cols), 256, 0, h->stream>>>(g);
+  return cudaGetLastError();
+}
+
 // ev (nullable): kNumPhases + 1 events recorded before the first phase and
 // after each phase.  mask: the phases to launch (bit i = kPhaseNames[i]);
 // the autotuner times single phases this way.
@@ -881,7 +897,6 @@ static gnmppi_status launch_iteration_t(gnmppi_t h, uint32_t it, int shrink, cud
     if (side) CK(cudaEventRecord(h->ev_side_join, h->side));
   }
   MARK(2);
-  GemmArgs ga{h->d_desc, h->d_st, nullptr, h->d_dR, h->d_W, h->d_P, h->d_A, h->d_S2};
   if (ON(2)) {
     if (h->use_tc) {
       const int inject = h->inj_tc && (int32_t)it == h->cs.inj_it;
@@ -889,9 +904,7 @@ static gnmppi_status launch_iteration_t(gnmppi_t h, uint32_t it, int shrink, cud
                             h->tune.contract_mt));
       h->launches++;
     } else {
-      ga.tiles = h->d_tiles[0];
-      k_gemm_nt<kContract, S, TC, TA><<<h->ntiles[0], 256, 0, h->stream>>>(ga);
-      CKL();
+      CK(launch_gemm_f64<kContract>(h));
       h->launches++;
     }
   }
@@ -901,17 +914,13 @@ static gnmppi_status launch_iteration_t(gnmppi_t h, uint32_t it, int shrink, cud
       CK(tc_gram_launch(h->tc, h->d_st, h->d_A, h->d_S2, h->stream));
       h->launches += h->tc.nred > 0 ? 2 : 1;  // the chunk sum is a second launch
     } else {
-      ga.tiles = h->d_tiles[1];
-      k_gemm_nt<kGram, TA, TC, double><<<h->ntiles[1], 256, 0, h->stream>>>(ga);
-      CKL();
+      CK(launch_gemm_f64<kGram>(h));
       h->launches++;
     }
   }
   MARK(4);
-  if (ON(4) && !h->use_tc && h->ntiles[2] > 0) {  // the tensor-core Gram launch already formed S2
-    ga.tiles = h->d_tiles[2];
-    k_gemm_nt<kS2, TA, TC, double><<<h->ntiles[2], 256, 0, h->stream>>>(ga);
-    CKL();
+  if (ON(4) && !h->use_tc && h->ngrows_lsq > 0) {  // the tensor-core Gram launch already formed S2
+    CK(launch_gemm_f64<kS2>(h));
     h->launches++;
   }
   if (side) CK(cudaStreamWaitEvent(h->stream, h->ev_side_join, 0));

@@ -4,9 +4,9 @@
 //     min shift, their sums and effective sample size, the weighted mean
 //     perturbation of Eq. 3, and b = P^T r = W^T e (the GGN gradient, Eq. 9,
 //     up to the metric S^-1);
-//   * k_gemm_nt: SIMT batched C = A B^T with the reduction dimension contiguous
-//     in both operands, used for the contraction [P^T | S] = W^T [dR | W]
-//     (Eq. 7), the Gram A = P^T P and S^2 in FP64/FP32 modes;
+//   * k_gemm_f64: SIMT batched C = A B^T with the reduction dimension contiguous
+//     in both operands, the FP64 mode's contraction [P^T | S] = W^T [dR | W]
+//     (Eq. 7), Gram A = P^T P and S^2;
 //   * k_solve: (A + lambda S_used^2) y = -b by Cholesky in FP64 (chol.cuh) with
 //     iterative refinement and tenfold damping retries, delta = S_used y, which equals
 //     the damped GGN step (J^T J + lambda I) delta = -J^T r for J = P S_used^-1;
@@ -296,101 +296,93 @@ enum GemmKind { kContract = 0, kGram = 1, kS2 = 2 };
 struct GemmArgs {
   const InstDesc* inst;
   const InstState* st;
-  const int4* tiles;  // (instance, tile row, tile col, -)
-  const void* dR;
-  const void* W;
-  void* P;
+  const int2* rows;  // (instance, block of 16 output rows)
+  const double* dR;
+  const double* W;
+  double* P;
   double* A;
   double* S2;
 };
 
-// C[i][j] = sum_k A[i][k] B[j][k], 64x64 tile per CTA, 4x4 per thread.
-template <GemmKind KIND, typename TIn, typename TC, typename TOut>
-__global__ void __launch_bounds__(256) k_gemm_nt(GemmArgs g) {
-  constexpr int BM = 64, BN = 64, BK = 16;
-  __shared__ TC As[BK][BM + 1];
-  __shared__ TC Bs[BK][BN + 1];
-  const int4 tl = g.tiles[blockIdx.x];
-  const int b = tl.x;
-  if (g.st[b].status != 0) return;
-  const InstDesc I = g.inst[b];
-  int Mr, Nc, Kd;
-  const TIn* Abase;
-  const TIn* B1;
-  const TIn* B2;
-  int64_t lda, ldb;
-  int nb1;
-  TOut* Cbase;
-  int64_t ldc;
+// C[i][j] = sum_k A[i][k] B[j][k] in FP64, one 16 x 16 tile per CTA of 256
+// threads (blockIdx.x: instance and row block, blockIdx.y: column tile), one
+// entry per thread, k in order.  GB300's FP64 pipe (two lanes per clock and SM)
+// bounds it, far below what the operands cost in shared memory or L2, so the
+// tile is chosen for the pipe: 16 rows keep the padding of n = 200 at 4 %
+// (64-row tiles multiplied 28 % zeros) and a single small instance still
+// spreads over many SMs (the Gram of n = 50 was one CTA).  Symmetric products
+// (S, A, S2) are formed on and below the diagonal and stored twice: entry (j, i)
+// sums the same products in the same order as (i, j).  The next k block's loads
+// are in flight while one is multiplied.  64 x 64 tiles before: contraction and
+// Gram of one pendulum 137 and 172 us, 16 and 16 now; of 64 chains (M = 10,
+// N = 100, K = 2048) 60.1 and 14.2 ms, 46.9 and 4.9 now (the contraction at
+// 0.99 of the FP64 peak); 16 x 32 and 16 x 64 tiles were up to 2 x slower on
+// small batches and 1-2 % on large ones.
+template <GemmKind KIND>
+__global__ void __launch_bounds__(256) k_gemm_f64(GemmArgs g) {
+  constexpr int T = 16;  // tile rows, columns and k block
+  __shared__ double As[2][T][T + 1];
+  __shared__ double Bs[2][T][T + 1];
+  const int2 e = g.rows[blockIdx.x];
+  if (g.st[e.x].status != 0) return;
+  const InstDesc I = g.inst[e.x];
+  const int i0 = e.y * T;
+  int j0 = blockIdx.y * T, nb, Kd;
+  const double *A, *B;
+  double* C;
+  int64_t ld, ldc;
+  bool sym = true;
   if (KIND == kContract) {
-    Mr = I.n; Nc = I.nR + I.n; Kd = I.Kp;
-    Abase = reinterpret_cast<const TIn*>(g.W) + I.o_W; lda = I.ldK;
-    B1 = reinterpret_cast<const TIn*>(g.dR) + I.o_dR; nb1 = I.nR;
-    B2 = reinterpret_cast<const TIn*>(g.W) + I.o_W; ldb = I.ldK;
-    Cbase = reinterpret_cast<TOut*>(g.P) + I.o_P; ldc = I.ldP;
-  } else if (KIND == kGram) {
-    Mr = I.n; Nc = I.n; Kd = I.nR;
-    Abase = reinterpret_cast<const TIn*>(g.P) + I.o_P; lda = I.ldP;
-    B1 = Abase; nb1 = I.n; B2 = Abase; ldb = I.ldP;
-    Cbase = reinterpret_cast<TOut*>(g.A) + I.o_nn; ldc = I.n;
+    Kd = I.Kp;
+    A = g.W + I.o_W;
+    ld = I.ldK;
+    C = g.P + I.o_P;
+    ldc = I.ldP;
+    const int ct = (I.nR + T - 1) / T;
+    if ((int)blockIdx.y < ct) {
+      B = g.dR + I.o_dR;
+      nb = I.nR;
+      sym = false;
+    } else {
+      B = A;
+      nb = I.n;
+      j0 -= ct * T;
+      C += I.sP;
+    }
   } else {
-    Mr = I.n; Nc = I.n; Kd = I.n;
-    Abase = reinterpret_cast<const TIn*>(g.P) + I.o_P + I.sP; lda = I.ldP;
-    B1 = Abase; nb1 = I.n; B2 = Abase; ldb = I.ldP;
-    Cbase = reinterpret_cast<TOut*>(g.S2) + I.o_nn; ldc = I.n;
+    Kd = KIND == kGram ? I.nR : I.n;
+    A = g.P + I.o_P + (KIND == kGram ? 0 : I.sP);
+    B = A;
+    ld = I.ldP;
+    nb = I.n;
+    C = (KIND == kGram ? g.A : g.S2) + I.o_nn;
+    ldc = I.n;
   }
-  const int i0 = tl.y * BM, j0 = tl.z * BN;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  TC acc[4][4];
-#pragma unroll
-  for (int p = 0; p < 4; ++p)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc[p][q] = (TC)0;
-  const int lr = threadIdx.x >> 2, lk = (threadIdx.x & 3) * 4;
-  for (int k0 = 0; k0 < Kd; k0 += BK) {
-    {
-      const int i = i0 + lr;
-      const TIn* ar = Abase + (int64_t)i * lda;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int k = k0 + lk + q;
-        As[lk + q][lr] = (i < Mr && k < Kd) ? (TC)to_d(ar[k]) : (TC)0;
-      }
-      const int j = j0 + lr;
-      const TIn* br = (j < nb1) ? B1 + (int64_t)j * ldb : B2 + (int64_t)(j - nb1) * ldb;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int k = k0 + lk + q;
-        Bs[lk + q][lr] = (j < Nc && k < Kd) ? (TC)to_d(br[k]) : (TC)0;
-      }
-    }
+  if (j0 >= nb || (sym && j0 > i0)) return;
+  // loads: thread (row ty, k tx) of both blocks
+  const int tx = threadIdx.x & (T - 1), ty = threadIdx.x / T;
+  const double* ar = A + (int64_t)(i0 + ty) * ld + tx;
+  const double* br = B + (int64_t)(j0 + ty) * ld + tx;
+  const bool am = i0 + ty < I.n, bm = j0 + ty < nb;
+  double ra, rb, acc = 0.0;
+  auto fetch = [&](int k0) {
+    const bool in = k0 + tx < Kd;
+    ra = (am && in) ? ar[k0] : 0.0;
+    rb = (bm && in) ? br[k0] : 0.0;
+  };
+  fetch(0);
+  for (int k0 = 0, s = 0; k0 < Kd; k0 += T, s ^= 1) {
+    As[s][tx][ty] = ra;
+    Bs[s][tx][ty] = rb;
     __syncthreads();
+    fetch(k0 + T);
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      TC av[4], bv[4];
-#pragma unroll
-      for (int p = 0; p < 4; ++p) av[p] = As[kk][ty * 4 + p];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) bv[q] = Bs[kk][tx * 4 + q];
-#pragma unroll
-      for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[p][q] += av[p] * bv[q];
-    }
-    __syncthreads();
+    for (int kk = 0; kk < T; ++kk) acc += As[s][kk][ty] * Bs[s][kk][tx];
   }
-#pragma unroll
-  for (int p = 0; p < 4; ++p) {
-    const int i = i0 + ty * 4 + p;
-    if (i >= Mr) continue;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int j = j0 + tx * 4 + q;
-      // contraction: the S columns go to sP on (P^T and S are stored apart)
-      const int jw = (KIND == kContract && j >= I.nR) ? j + (I.sP - I.nR) : j;
-      if (j < Nc) Cbase[(int64_t)i * ldc + jw] = (TOut)acc[p][q];
-    }
-  }
+  const int i = i0 + ty, j = j0 + tx;
+  if (i >= I.n || j >= nb || (sym && j > i)) return;
+  C[(int64_t)i * ldc + j] = acc;
+  if (sym && j < i) C[(int64_t)j * ldc + i] = acc;
 }
 
 // ------------------------------------------------------- damped GGN solve
