@@ -16,26 +16,28 @@ namespace gnm {
 // FX > 0: the chain has exactly FX free masses, known at compile time, so
 // that the "slot holds a real mass" and "slot holds the forced mass" tests
 // fold to constants for every slot but the last lanes' (FX = 0: F at run time).
+// This form is FP64 (FP32 below).
 template <typename T, int FL, int G, int FX = 0>
 struct ChainGroup {
+  static_assert(sizeof(T) == 8, "the FP32 group chain is the specialisation below");
   static constexpr int NXL = 4 * FL;  // lane-local state: p (2FL), v (2FL)
   static constexpr bool kRelative = false;  // positions are absolute
-  T mass_inv, k, k3, c, g, l0, h, h2, h6;
+  T mass_inv, km, k3m, cm, g, l0, h, h2, h6;
   int F, lg;
   unsigned mask;  // lanes that execute this group's shuffles together
   const T* pref;  // target positions: global row indexed (pref_local false) or lane-local (2FL)
   bool pref_local;
   __device__ ChainGroup(const Consts& cs, int F_, int lg_, unsigned mask_)
       : F(F_), lg(lg_), mask(mask_), pref(nullptr), pref_local(false) {
-    mass_inv = (T)(1.0 / cs.params[0]);
-    k = (T)cs.params[1];
-    k3 = (T)cs.params[2];
-    c = (T)cs.params[3];
-    g = (T)cs.params[4];
-    l0 = (T)(1.0 / (double)F_);
-    h = (T)cs.dt;
-    h2 = (T)(0.5 * cs.dt);
-    h6 = (T)(cs.dt / 6.0);
+    mass_inv = 1.0 / cs.params[0];
+    km = cs.params[1] / cs.params[0];
+    k3m = cs.params[2] / cs.params[0];
+    cm = -cs.params[3] / cs.params[0];
+    g = cs.params[4];
+    l0 = 1.0 / (double)F_;
+    h = cs.dt;
+    h2 = 0.5 * cs.dt;
+    h6 = cs.dt / 6.0;
   }
   __device__ __forceinline__ int mass(int j) const { return lg * FL + j + 1; }  // 1-based global index
   // slot j of this lane holds a real mass / the mass the control force acts on
@@ -44,58 +46,49 @@ struct ChainGroup {
     return FX > 0 ? (j == (FX - 1) % FL && lg == (FX - 1) / FL) : mass(j) == F;
   }
   __device__ __forceinline__ void set_reference(const double*) {}
-  __device__ __forceinline__ void accel(const T* s, const T* u, T* acc) const {
+  __device__ __forceinline__ void accel(const T* s, const T* um, T* acc) const {
     const T* v = s + 2 * FL;
     // position of the mass before this lane's first one (origin for lane 0)
     T pxp = __shfl_up_sync(mask, s[2 * (FL - 1)], 1, G);
     T pyp = __shfl_up_sync(mask, s[2 * (FL - 1) + 1], 1, G);
     if (lg == 0) pxp = pyp = (T)0;
-    T fx[FL], fy[FL];
+    // link j of this lane ends at its mass j: vector and force scale (common.cuh)
+    T dx[FL], dy[FL], fr[FL];
 #pragma unroll
     for (int j = 0; j < FL; ++j) {
-      const T px0 = (j == 0) ? pxp : s[2 * (j - 1)];
-      const T py0 = (j == 0) ? pyp : s[2 * (j - 1) + 1];
-      const T dx = s[2 * j] - px0;
-      const T dy = s[2 * j + 1] - py0;
+      dx[j] = s[2 * j] - ((j == 0) ? pxp : s[2 * (j - 1)]);
+      dy[j] = s[2 * j + 1] - ((j == 0) ? pyp : s[2 * (j - 1) + 1]);
       const bool real = this->real(j);
-      const T q = real ? dx * dx + dy * dy : (T)1;
-      if constexpr (sizeof(T) == 4) {
-        const T rinv = rsqrtf(q);
-        const T dd = q * rinv - l0;
-        const T fr = real ? (k * dd + k3 * dd * dd * dd) * rinv : (T)0;
-        fx[j] = fr * dx;
-        fy[j] = fr * dy;
-      } else {
-        const T len = sqrt(q);
-        const T dd = len - l0;
-        const T fm = real ? k * dd + k3 * dd * dd * dd : (T)0;
-        fx[j] = fm * dx / len;
-        fy[j] = fm * dy / len;
-      }
+      const T q = real ? fma(dx[j], dx[j], dy[j] * dy[j]) : (T)1;
+      const T f = link_scale(q, l0, km, k3m);
+      fr[j] = real ? f : (T)0;
     }
-    // force of the link after this lane's last mass (first link of the next lane)
-    T fxn = __shfl_down_sync(mask, fx[0], 1, G);
-    T fyn = __shfl_down_sync(mask, fy[0], 1, G);
-    if (lg == G - 1) fxn = fyn = (T)0;
+    // the next lane's first link (the one after this lane's last mass)
+    const T dxn = __shfl_down_sync(mask, dx[0], 1, G);
+    const T dyn = __shfl_down_sync(mask, dy[0], 1, G);
+    T frn = __shfl_down_sync(mask, fr[0], 1, G);
+    if (lg == G - 1) frn = (T)0;
 #pragma unroll
     for (int j = 0; j < FL; ++j) {
-      const T nx = (j + 1 < FL) ? fx[j + 1] : fxn;
-      const T ny = (j + 1 < FL) ? fy[j + 1] : fyn;
-      T ax = -c * v[2 * j] - fx[j] + nx;
-      T ay = -c * v[2 * j + 1] - fy[j] + ny;
+      const T fo = (j + 1 < FL) ? fr[j + 1] : frn;
+      T ax = fma(-fr[j], dx[j], cm * v[2 * j]);
+      T ay = fma(-fr[j], dy[j], fma(cm, v[2 * j + 1], -g));
+      ax = fma(fo, (j + 1 < FL) ? dx[j + 1] : dxn, ax);
+      ay = fma(fo, (j + 1 < FL) ? dy[j + 1] : dyn, ay);
       if (ctrl(j)) {
-        ax += u[0];
-        ay += u[1];
+        ax += um[0];
+        ay += um[1];
       }
       const bool real = this->real(j);
-      acc[2 * j] = real ? ax * mass_inv : (T)0;
-      acc[2 * j + 1] = real ? ay * mass_inv - g : (T)0;
+      acc[2 * j] = real ? ax : (T)0;
+      acc[2 * j + 1] = real ? ay : (T)0;
     }
   }
   __device__ __forceinline__ void step(T* x, const T* u) const {
     constexpr int H = 2 * FL;
     T a[NXL], t[NXL], acc[H];
-    accel(x, u, acc);
+    const T um[2] = {u[0] * mass_inv, u[1] * mass_inv};
+    accel(x, um, acc);
 #pragma unroll
     for (int i = 0; i < H; ++i) {
       a[i] = x[H + i];
@@ -103,7 +96,7 @@ struct ChainGroup {
       t[i] = x[i] + h2 * x[H + i];
       t[H + i] = x[H + i] + h2 * acc[i];
     }
-    accel(t, u, acc);
+    accel(t, um, acc);
 #pragma unroll
     for (int i = 0; i < H; ++i) {
       a[i] = a[i] + (T)2 * t[H + i];
@@ -111,7 +104,7 @@ struct ChainGroup {
       t[i] = x[i] + h2 * t[H + i];
       t[H + i] = x[H + i] + h2 * acc[i];
     }
-    accel(t, u, acc);
+    accel(t, um, acc);
 #pragma unroll
     for (int i = 0; i < H; ++i) {
       a[i] = a[i] + (T)2 * t[H + i];
@@ -119,7 +112,7 @@ struct ChainGroup {
       t[i] = x[i] + h * t[H + i];
       t[H + i] = x[H + i] + h * acc[i];
     }
-    accel(t, u, acc);
+    accel(t, um, acc);
 #pragma unroll
     for (int i = 0; i < H; ++i) {
       x[i] = x[i] + h6 * (a[i] + t[H + i]);
