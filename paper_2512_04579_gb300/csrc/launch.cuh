@@ -37,7 +37,7 @@ cudaError_t prepare_samples(int smem) {
 }
 template <class Model, typename T>
 void launch_line(const RollArgs& a, int nthreads, cudaStream_t s) {
-  if (nthreads > 0) k_line<Model, T><<<(nthreads + 127) / 128, 128, 0, s>>>(a);
+  if (nthreads > 0) k_line<Model, T><<<(nthreads + 31) / 32, 32, 0, s>>>(a);
 }
 
 template <class M32, class M64, typename T, typename S>
@@ -54,6 +54,10 @@ void fill(Launchers* o) {
 // shorter (same rows and costs, see k_line_group).  Measured at 256 chain
 // instances (16 candidates each): M = 10 0.18 / 0.127 / 0.096 / 0.105 ms with
 // 1 / 4 / 8 / 16 lanes per candidate, M = 16 0.152 / 0.094 / 0.107 ms with 4 / 8 / 16.
+// Two warps per CTA: a candidate's rollout is one serial chain, so a batch's
+// few warps belong on as many SM sub-partitions as there are (256-thread CTAs
+// put eight on one SM: 16 chains of M = 32 258 us, 138 now; eight FP64 chains
+// of M = 10 2.10 ms, 1.08 now; 256 chains of M = 10 84, 82 us).
 template <typename T, int FL, int G, int FX = 0>
 void launch_line_group(const RollArgs& a, int ncand_total, cudaStream_t s) {
   const long lanes = (long)ncand_total * G;
@@ -62,9 +66,9 @@ void launch_line_group(const RollArgs& a, int ncand_total, cudaStream_t s) {
   // lane-parallel over the steps) in shared memory when they fit the default
   // 48 KB; longer horizons form them per step
   RollArgs b = a;
-  const size_t smem = (size_t)(256 / G) * (size_t)a.nmax * sizeof(float2);
+  const size_t smem = (size_t)(kLineGroupThreads / G) * (size_t)a.nmax * sizeof(float2);
   b.pre = (sizeof(T) == 4 && a.mode != 2 && smem <= 48 * 1024) ? 1 : 0;
-  k_line_group<T, FL, G, FX><<<(unsigned)((lanes + 255) / 256), 256, b.pre ? smem : 0, s>>>(b);
+  k_line_group<T, FL, G, FX><<<(unsigned)((lanes + kLineGroupThreads - 1) / kLineGroupThreads), kLineGroupThreads, b.pre ? smem : 0, s>>>(b);
 }
 template <typename T, typename S, int F>
 void fill_chain(Launchers* o) {

@@ -280,11 +280,13 @@ struct LineEmit {
   }
 };
 
-// One thread per (instance, candidate).  mode 0: candidate j rolls out
+// One thread per (instance, candidate), one warp per CTA: a rollout is one
+// serial chain, so the few warps of a small batch go to as many SMs (128-thread
+// CTAs: 64 chains of M = 4 172 us, 123 now).  mode 0: candidate j rolls out
 // U + gamma^j delta; mode 1: the nominal U; mode 2: the nominal U in FP64 into
 // Cout.  Instances whose status is not OK are skipped.
 template <class Model, typename T>
-__global__ void __launch_bounds__(128) k_line(RollArgs a) {
+__global__ void __launch_bounds__(32) k_line(RollArgs a) {
   constexpr int NX = Model::NX, NU = Model::NU;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int ncand = a.mode == 0 ? a.ncand : 1;

@@ -452,8 +452,12 @@ __global__ void __launch_bounds__(256, 2) k_samples_group(RollArgs a) {
 }
 
 // Line search / nominal / FP64 cost for groups: one group per (instance, candidate).
+// The 64-thread launch bound pays for lanes of four and more masses (M = 32, 16
+// instances: 138 -> 125 us; M = 64: 135 -> 121), not for two (M = 10, 256
+// instances: 82 -> 86).
+constexpr int kLineGroupThreads = 64;
 template <typename T, int FL, int G, int FX = 0>
-__global__ void __launch_bounds__(256) k_line_group(RollArgs a) {
+__global__ void __launch_bounds__(FL >= 4 ? kLineGroupThreads : 256) k_line_group(RollArgs a) {
   const int gid = (int)((blockIdx.x * blockDim.x + threadIdx.x) / G);
   const int lg = threadIdx.x & (G - 1);
   const int ncand = a.mode == 0 ? a.ncand : 1;
