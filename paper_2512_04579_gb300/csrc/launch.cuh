@@ -24,6 +24,10 @@ bool group_launchers_f32(int F, Launchers* out);
 
 template <class Model, typename T, typename S>
 void launch_samples(const RollArgs& a, int nb, int smem, cudaStream_t s) {
+  if (sizeof(T) == 8 && a.cs.sampling == 0) {
+    const dim3 grid((unsigned)nb, (unsigned)((a.nmax * Model::NU + 1) / 2));
+    k_noise_f64<<<grid, a.cs.antithetic ? kPairsPerBlock : kSamplesPerBlock, 0, s>>>(a);
+  }
   if (a.cs.antithetic)
     k_samples<Model, T, S, true><<<nb, 128, smem, s>>>(a);
   else

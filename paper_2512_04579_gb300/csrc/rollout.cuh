@@ -125,6 +125,27 @@ struct SampleEmit {
   }
 };
 
+// FP64: the perturbations W = s z of the blocks of k_samples, written to W one
+// Box-Muller pair per thread (blockIdx.y: normals 2q and 2q + 1), before the
+// rollouts read them.  A log, a square root and a sine / cosine pair are some
+// hundred FP64 instructions, one per warp per 64 cycles on GB300; inside the
+// rollouts both lanes of an antithetic pair ran them in their one serial chain;
+// here every pair of normals has a thread of its own (pendulum, N = 50, K = 256:
+// both kernels 259 us, 308 before; 64 instances 287, 310 before; chain M = 10
+// 4.72 ms, 4.83 before).
+static __global__ void __launch_bounds__(128) k_noise_f64(RollArgs a) {
+  const int2 bm = a.bmap[blockIdx.x];
+  const InstDesc I = a.inst[bm.x];
+  const int m = bm.y * (int)blockDim.x + threadIdx.x, j = 2 * blockIdx.y;
+  if (a.st[bm.x].status != 0 || m >= I.Kp || j >= I.n) return;
+  double z0, z1;
+  box_muller(noise_words(a.cs.seed, (uint32_t)(bm.x + a.cs.inst_base), a.it, (uint32_t)m, (uint32_t)blockIdx.y), z0, z1);
+  double* W = reinterpret_cast<double*>(a.W) + I.o_W + (int64_t)j * I.ldK + m;
+  const double* s = a.s + I.o_U + j;
+  if (GNM_IN(j, I.n)) W[0] = s[0] * z0;
+  if (j + 1 < I.n && GNM_IN(j + 1, I.n)) W[I.ldK] = s[1] * z1;
+}
+
 template <class Model, typename T, typename S, bool ANTI>
 __global__ void __launch_bounds__(128) k_samples(RollArgs a) {
   constexpr int NX = Model::NX, NU = Model::NU;
@@ -174,6 +195,11 @@ __global__ void __launch_bounds__(128) k_samples(RollArgs a) {
   // Sigma points (Method E): pair m perturbs control m alone, by sqrt(n) s_m.
   const bool sigma_pts = ANTI && a.cs.sampling != 0;
   const T sqrtn = sqrt((T)I.n);
+  // FP64 reads the perturbations that k_noise_f64 wrote, a step ahead
+  constexpr bool READ = sizeof(T) == 8;
+  T wn[NU];
+#pragma unroll
+  for (int c = 0; c < NU; ++c) wn[c] = (READ && !sigma_pts && active) ? (T)Wm[(int64_t)c * I.ldK + m] : (T)0;
   int qc = -1;
   T z0 = (T)0, z1 = (T)0, y0 = (T)0, y1 = (T)0;
   for (int k = 0; k < I.N; ++k) {
@@ -185,6 +211,13 @@ __global__ void __launch_bounds__(128) k_samples(RollArgs a) {
         const T w = (j == m) ? sS[j] * sqrtn : (T)0;
         u[c] = sU[j] + sign * w;
         if (active && par == 0 && GNM_IN(j, I.n)) put_w(Wm, W2b, I.ldK, j, m, w);
+      }
+    } else if (READ) {
+#pragma unroll
+      for (int c = 0; c < NU; ++c) {
+        const int j = k * NU + c;
+        u[c] = sU[j] + sign * wn[c];
+        wn[c] = (active && k + 1 < I.N) ? (T)Wm[(int64_t)(j + NU) * I.ldK + m] : (T)0;
       }
     } else if (SHARE) {
       if ((k & 1) == 0) {
