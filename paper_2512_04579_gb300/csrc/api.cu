@@ -563,6 +563,7 @@ static gnmppi_status build(gnmppi_t h, const gnmppi_instance_shape* shapes) {
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     h->tune.solve_nt = h->batch <= nsm ? 512 : 256;
+    if (h->use_tc && prec == kBF16) h->tune.contract_mt = tc_contract_default_mt(h->tc, nsm);
   }
   set_branches(h, std::min<int>(4, (int)h->groups.size()));
   CK(cudaStreamSynchronize(h->stream));
@@ -863,7 +864,8 @@ static gnmppi_status launch_iteration_t(gnmppi_t h, uint32_t it, int shrink, cud
       a.bmap = g.d_bmap;
       g.fn.samples(a, (int)g.bmap.size(), g.smem, s);
       CKL();
-      h->launches++;
+      // the FP64 thread-per-rollout chains' noise is a launch of its own
+      h->launches += (h->p.precision == kFP64 && !g.fn.pairs_per_block && !h->p.sampling) ? 2 : 1;
       return GNMPPI_OK;
     });
     if (st != GNMPPI_OK) return st;

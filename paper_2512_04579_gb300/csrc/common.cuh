@@ -204,16 +204,16 @@ __device__ __forceinline__ void put(float* p, float v) { *p = v; }
 
 // Sample m of row j of the BF16 mode's split copy of W: the BF16 head of w
 // (round to nearest even) and the BF16 rounding of its remainder w - head,
-// laid out per 16 samples as 16 heads then 16 remainders (one 64-byte row of
+// laid out per 32 samples as 32 heads then 32 remainders (one 128-byte row of
 // the contraction's BF16 operand for that k-block).  row: the copy's row j,
 // ldK words = 2 ldK BF16 slots.  The same arithmetic as the contraction's
 // in-place split of FP32 W rows.
 __device__ __forceinline__ void put_w2(uint16_t* row, int m, float w) {
   const __nv_bfloat16 h = __float2bfloat16_rn(w);
   const __nv_bfloat16 l = __float2bfloat16_rn(w - __bfloat162float(h));
-  const int i = (m >> 4) * 32 + (m & 15);
+  const int i = (m >> 5) * 64 + (m & 31);
   row[i] = __bfloat16_as_ushort(h);
-  row[i + 16] = __bfloat16_as_ushort(l);
+  row[i + 32] = __bfloat16_as_ushort(l);
 }
 
 __device__ __forceinline__ double to_d(double x) { return x; }

@@ -13,11 +13,11 @@
 //      rows of the [dR; W] block (two 128-row sub-tiles, each with its own
 //      256-column TMEM accumulator) with up to 256 W rows, from three
 //      kind::f16 passes per product:
-//        warp 0 lane 0  issues TMA loads of 16-value k-blocks into a 6-stage
+//        warp 0 lane 0  issues TMA loads of 32-value k-blocks into a 3-stage
 //                       ring: the FP32 [dR; W] rows, and the W rows from the
 //                       rollouts' BF16 head/remainder copy of W,
-//        warps 2-5      rewrite each landed FP32 row in place as a BF16
-//                       [head | remainder] row (each thread its own rows),
+//        warps 2-9      rewrite each landed FP32 row in place as a BF16
+//                       [head | remainder] row (each thread one row),
 //        warp 1 lane 0  issues tcgen05.mma (M=128, N = the W rows, K=16) per
 //                       sub-tile,
 //        warps 0-3      read TMEM back (tcgen05.ld 32x32b, one lane per
@@ -30,10 +30,10 @@
 //      launch S2 = S S^T for the scaled LSQ system.  FP32 mode: TF32 heads
 //      h = rna(x) (remainder exact in FP32), 32-value k-blocks, the remainder
 //      beside the head.  BF16 mode: BF16 head and remainder written in place
-//      as a [head | remainder] row per 16-value k-block, as in (1), one
+//      as a [head | remainder] row per 32-value k-block, as in (1), one
 //      128-row sub-tile per CTA and two CTAs per SM.  TMA
 //      streams the FP32 rows of [P^T | S] straight from the contraction's
-//      output; warps 2-5 split each landed stage in shared memory before the
+//      output; warps 2-9 split each landed stage in shared memory before the
 //      MMAs read it.  A
 //      diagonal tile takes its A sub-tiles from its own B rows (the operand is
 //      the same matrix), each sub-tile's MMAs stop at the diagonal, and the
@@ -56,8 +56,7 @@ namespace {
 
 constexpr int BM = 128, BN = 256;
 constexpr int ROW_BYTES = 128;  // one k-block of an FP32 row: 32 values
-constexpr int KBLK_F32 = 32;    // Gram and three-pass TF32 k-block (128-byte rows, 128-byte swizzle)
-constexpr int KBLK_BF16 = 16;   // BF16-mode contraction k-block (64-byte rows, 64-byte swizzle)
+constexpr int KBLK = 32;        // k-block: 32 FP32 values, or their 32 BF16 heads and 32 remainders
 constexpr int A_BYTES = BM * ROW_BYTES;
 constexpr int B_BYTES = BN * ROW_BYTES;
 constexpr int RING_BYTES = 4 * (A_BYTES + B_BYTES);  // 192 KB of operand ring (every kernel here)
@@ -74,37 +73,34 @@ __device__ __forceinline__ void bf16_split2(float a, float b, uint32_t& hi, uint
   lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
-// Row `row` of a landed 64-byte-swizzled TMA box at p (16 FP32 values, one
-// contraction k-block) rewritten in place as a 64-byte BF16 row [16 heads |
-// 16 remainders] with the same swizzle (16-byte chunk j of the row at chunk
-// j ^ ((row >> 1) & 3)).  The row's four chunks are read before any is
-// written and no other row's bytes are touched, so each thread splits its
-// own rows without waiting for the others.
-__device__ __forceinline__ void split_row_sw64(unsigned char* p, int row) {
-  unsigned char* r = p + row * 64;
-  const int sw = (row >> 1) & 3;
-  float v[16];
+// Row `row` of a landed 128-byte-swizzled TMA box at p (32 FP32 values, one
+// k-block) rewritten in place as a 128-byte BF16 row [32 heads | 32
+// remainders] with the same swizzle (16-byte chunk j of the row at chunk
+// j ^ (row & 7)).  The row's chunks are read before any is written and no
+// other row's bytes are touched, so each thread splits its own rows without
+// waiting for the others.
+__device__ __forceinline__ void split_row(unsigned char* p, int row) {
+  unsigned char* r = p + row * ROW_BYTES;
+  const int sw = row & 7;
+  float v[32];
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
+  for (int c = 0; c < 8; ++c) {
     const float4 q = *reinterpret_cast<const float4*>(r + ((c ^ sw) << 4));
     v[4 * c] = q.x;
     v[4 * c + 1] = q.y;
     v[4 * c + 2] = q.z;
     v[4 * c + 3] = q.w;
   }
-  uint4 H0, L0, H1, L1;  // heads of values 0-7 and 8-15, remainders likewise
-  bf16_split2(v[0], v[1], H0.x, L0.x);
-  bf16_split2(v[2], v[3], H0.y, L0.y);
-  bf16_split2(v[4], v[5], H0.z, L0.z);
-  bf16_split2(v[6], v[7], H0.w, L0.w);
-  bf16_split2(v[8], v[9], H1.x, L1.x);
-  bf16_split2(v[10], v[11], H1.y, L1.y);
-  bf16_split2(v[12], v[13], H1.z, L1.z);
-  bf16_split2(v[14], v[15], H1.w, L1.w);
-  *reinterpret_cast<uint4*>(r + ((0 ^ sw) << 4)) = H0;
-  *reinterpret_cast<uint4*>(r + ((1 ^ sw) << 4)) = H1;
-  *reinterpret_cast<uint4*>(r + ((2 ^ sw) << 4)) = L0;
-  *reinterpret_cast<uint4*>(r + ((3 ^ sw) << 4)) = L1;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {  // heads and remainders of values 8 c .. 8 c + 7
+    uint4 H, L;
+    bf16_split2(v[8 * c], v[8 * c + 1], H.x, L.x);
+    bf16_split2(v[8 * c + 2], v[8 * c + 3], H.y, L.y);
+    bf16_split2(v[8 * c + 4], v[8 * c + 5], H.z, L.z);
+    bf16_split2(v[8 * c + 6], v[8 * c + 7], H.w, L.w);
+    *reinterpret_cast<uint4*>(r + ((c ^ sw) << 4)) = H;
+    *reinterpret_cast<uint4*>(r + (((c + 4) ^ sw) << 4)) = L;
+  }
 }
 
 // One (128 or 256) x (up to 256) tile of the BF16 mode's contraction: the A
@@ -113,33 +109,42 @@ __device__ __forceinline__ void split_row_sw64(unsigned char* p, int row) {
 // D[i][j] = sum_k A[i][k] B[j][k] is stored transposed, into row j and column
 // i of [P^T | S] (columns >= ccut cgap further right): one TMEM lane per
 // output column i, so each warp store writes 32 consecutive columns.  TMA
-// lands k-blocks of 16 values (64-byte rows, 64-byte swizzle): the FP32 rows
-// of up to two 128-row A sub-tiles, which four splitter warps rewrite in
-// place as BF16 [head | remainder] rows, and 256 B rows from the rollouts'
+// lands k-blocks of 32 values (128-byte rows and swizzle): the FP32 rows of up
+// to two 128-row A sub-tiles, which the splitter threads rewrite in place, one
+// row each, as BF16 [head | remainder] rows, and 256 B rows from the rollouts'
 // BF16 copy of W, which arrive in that layout already (split once per
 // iteration instead of once per tile).  Each product is formed from three
 // BF16 MMAs of K = 16 (head x head, head x remainder, remainder x head, the
-// remainders 32 bytes into the rows), which keeps FP32-level accuracy (the
-// dropped remainder x remainder term is ~2^-18 relative).  192 threads: warp
-// 0 lane 0 TMA, warp 1 lane 0 MMA, warps 2-5 split; warps 0-3 read TMEM back.
+// remainders 64 bytes into the rows), which keeps FP32-level accuracy (the
+// dropped remainder x remainder term is ~2^-18 relative).  Warp 0 lane 0 TMA,
+// warp 1 lane 0 MMA, warps 2 on split; warps 0-3 read TMEM back.
 //
-// MT: A sub-tiles per CTA.  MT = 2: 256 A rows, a 6-stage ring of 32 KB, one
-// CTA per SM; MT = 1: 128 A rows, a 4-stage ring of 24 KB (96 KB), two CTAs per
-// SM, whose pipelines hide each other's load latency (the W rows are then read
-// twice as often, from L2).  Same products, same accumulation order per output.
-constexpr int kContractThreads = 192;
+// What bounds a tile is shared memory's 128 bytes per clock: per k-block the
+// TMA fill (64 KB), the A rows' split (32 + 32 KB) and the MMAs' operand reads
+// (12 x 10.6 KB), about 2000 cycles; about 1800 are spent.  k-blocks of 16
+// values (64-byte rows) took 1450 each: half-width TMA rows and twice the
+// barriers (256 chains of M = 10, K = 2048: 0.72 ms, 0.66 now; one: 47 us, 39
+// now; DRAM's floor at 256 is 0.44 ms).  Four splitter warps with two rows per
+// thread took as long as eight.
+//
+// MT: A sub-tiles per CTA.  MT = 2: 256 A rows, a 3-stage ring of 64 KB, one
+// CTA per SM; MT = 1: 128 A rows, a 2-stage ring of 48 KB, two CTAs per SM, one
+// of which loads while the other starts up or stores (the W rows are then read
+// twice as often, from L2).  Same products, same accumulation order per
+// output.  tc_contract_default_mt() has the default's rule.
 template <int MT>
-__global__ void __launch_bounds__(kContractThreads, 3 - MT) k_contract_tc(const CUtensorMap* __restrict__ maps,
+constexpr int kContractThreads = 64 + MT * BM;
+template <int MT>
+__global__ void __launch_bounds__(kContractThreads<MT>, 3 - MT) k_contract_tc(const CUtensorMap* __restrict__ maps,
                                                                     const TcJob* __restrict__ jobs,
                                                                     const InstState* __restrict__ st,
                                                                     const int4* __restrict__ tiles,
                                                                     float* __restrict__ D, int* __restrict__ err,
                                                                     int inject) {
-  constexpr int KBLK = KBLK_BF16;            // FP32 values per k-block (one 64-byte row)
-  constexpr int TILE = BM * 64;              // one landed 128-row box (8 KB)
+  constexpr int TILE = A_BYTES;              // one landed 128-row box (16 KB)
   constexpr int STAGE_BYTES = (MT + 2) * TILE;  // A sub-tiles, then 256 B rows
   constexpr int STAGES = (MT == 2 ? RING_BYTES : RING_BYTES / 2) / STAGE_BYTES;
-  constexpr int SPLITTERS = kContractThreads - 64;
+  constexpr int SPLITTERS = MT * BM;
   constexpr uint32_t TCOLS = MT * TMEM_COLS;
   const int4 tl = tiles[blockIdx.x];
   const TcJob J = jobs[tl.x];
@@ -221,7 +226,7 @@ __global__ void __launch_bounds__(kContractThreads, 3 - MT) k_contract_tc(const 
         break;
       }
       unsigned char* sb = base + s * STAGE_BYTES;
-      for (int q = 0; q < mt; ++q) split_row_sw64(sb + q * TILE, t);
+      if (MT == 1 || (t >> 7) < mt) split_row(sb + (t >> 7) * TILE, t & 127);
       // the generic-proxy writes become visible to the tensor core's reads
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(bars + STAGES + s)) : "memory");
@@ -247,14 +252,17 @@ __global__ void __launch_bounds__(kContractThreads, 3 - MT) k_contract_tc(const 
       }
       tc_fence_after();
       const uint32_t a0 = su32(base + s * STAGE_BYTES);
-      const uint32_t bh = a0 + MT * TILE, bl = bh + 32;
       // sub-tile q accumulates into TMEM columns [256 q, 256 q + 256)
       for (int q = 0; q < mt; ++q) {
         const uint32_t d = tmem + (uint32_t)(q * TMEM_COLS);
-        const uint32_t ah = a0 + q * TILE, al = ah + 32;
-        mma<true>(d, sdesc<true>(ah), sdesc<true>(bh), id, kb > 0 ? 1u : 0u);
-        mma<true>(d, sdesc<true>(ah), sdesc<true>(bl), id, 1u);
-        mma<true>(d, sdesc<true>(al), sdesc<true>(bh), id, 1u);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {  // 16 values per MMA; the remainders 64 bytes into the rows
+          const uint32_t ah = a0 + q * TILE + k * 32, al = ah + 64;
+          const uint32_t bh = a0 + MT * TILE + k * 32, bl = bh + 64;
+          mma<true>(d, sdesc(ah), sdesc(bh), id, (kb > 0 || k > 0) ? 1u : 0u);
+          mma<true>(d, sdesc(ah), sdesc(bl), id, 1u);
+          mma<true>(d, sdesc(al), sdesc(bh), id, 1u);
+        }
       }
       mma_commit(su32(bars + 2 * STAGES + s));  // frees the stage once these MMAs have read it
     }
@@ -285,7 +293,7 @@ __global__ void __launch_bounds__(kContractThreads, 3 - MT) k_contract_tc(const 
         tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(sub * TMEM_COLS + c * 32), v);
         const int j0 = tl.z * BN + c * 32;
         if (live) {
-#pragma unroll 8
+#pragma unroll
           for (int jj = 0; jj < 32; ++jj)
             if (c * 32 + jj < jn && GNM_IN((int64_t)(j0 + jj) * J.ldc + colw, (int64_t)J.M * J.ldc))
               out[(int64_t)(j0 + jj) * J.ldc + colw] = __uint_as_float(v[jj]);
@@ -381,25 +389,23 @@ __device__ __forceinline__ void store_block(T* out, const T* stg, const TcJob& J
 // Gram tile of one job: output rows tl.y.., columns tl.z.. (the B rows),
 // tl.w = sub-tiles (1 or 2) | 4 if the tile sits on the diagonal.  Per stage
 // (one 32-column k-block): B head and remainder (256 rows), and for an
-// off-diagonal tile A head and remainder (128 rows).  192 threads: warp 0
-// lane 0 TMA, warp 1 lane 0 MMA, warps 2-5 split; warps 0-3 read TMEM back.
+// off-diagonal tile A head and remainder (128 rows).  Warp 0 lane 0 TMA, warp
+// 1 lane 0 MMA, warps 2-9 split; warps 0-3 read TMEM back.
 // CONTRACT: the same three-pass product for the FP32 mode's contraction
 // [P^T | S] = W^T [dR | W] (off-diagonal tiles only, A rows a_row0 + i and B
 // rows b_row0 + j of the instance's FP32 [dR; W] map), FP32 output into out0
 // with the S columns moved to sP; otherwise A = out0 or S2 in FP64.
-constexpr int kGramThreads = 192;
-// BF (the BF16 mode's Gram, CONTRACT false only): k-blocks of 16 FP32 values
-// (64-byte rows, 64-byte swizzle) split in place row by row into BF16
-// [head | remainder] rows, three kind::f16 passes; B rows and (off the
-// diagonal) A rows only, no separate remainder area.  Every tile has one
-// 128-row sub-tile (256 TMEM columns) and a 96 KB ring (up to 8 stages), so
+constexpr int kGramThreads = 64 + 2 * BM;
+// BF (the BF16 mode's Gram, CONTRACT false only): k-blocks split in place row
+// by row into BF16 [head | remainder] rows, three kind::f16 passes; B rows and
+// (off the diagonal) A rows only, no separate remainder area.  Every tile has
+// one 128-row sub-tile (256 TMEM columns) and a 96 KB ring (up to 6 stages), so
 // two CTAs share an SM and each hides the other's pipeline latency: a
 // diagonal tile with two sub-tiles runs as two CTAs (tl.w bit 3 marks the
 // second), the first loading only the 128 B rows its MMAs read.  Same
 // products in the same order per output as one CTA per diagonal tile
-// (0.266 -> 0.215 ms per launch at 256 instances of n = 200).  12 diagonal
-// stages of 16 KB in a 192 KB ring measured slower (0.92 against 0.84 ms for
-// 64 instances of M = 32).
+// (0.266 -> 0.215 ms per launch at 256 instances of n = 200).  k-blocks of 16
+// values took 90 us for one chain of M = 10, 74 now, and as long for 256.
 template <bool CONTRACT, bool BF = false>
 __global__ void __launch_bounds__(kGramThreads, BF ? 2 : 1) k_gram_tc(const CUtensorMap* __restrict__ maps, const TcJob* __restrict__ jobs,
                                                     const InstState* __restrict__ st, const int4* __restrict__ tiles,
@@ -408,11 +414,10 @@ __global__ void __launch_bounds__(kGramThreads, BF ? 2 : 1) k_gram_tc(const CUte
                                                     int* __restrict__ err, int inject) {
   using TO = typename std::conditional<CONTRACT, float, double>::type;
   static_assert(!(CONTRACT && BF), "the BF16 contraction is k_contract_tc");
-  // FP32 elements per k-block; MMAs (TF32 K = 8, BF16 K = 16) per k-block
-  constexpr int KBLK = BF ? KBLK_BF16 : 32, NSUB = BF ? 1 : 4;
-  constexpr int RB = BF ? 64 : ROW_BYTES;  // bytes of one landed row of a k-block
-  constexpr int SPLITTERS = kGramThreads - 64;  // warps 2-5
-  constexpr int MAXST = BF ? 8 : 3;
+  constexpr int NSUB = BF ? 2 : 4;  // MMAs (TF32 K = 8, BF16 K = 16) per k-block
+  constexpr int RB = ROW_BYTES;  // bytes of one landed row of a k-block
+  constexpr int SPLITTERS = kGramThreads - 64;  // warps 2-9
+  constexpr int MAXST = BF ? 6 : 3;
   const int4 tl = tiles[blockIdx.x];
   const TcJob J = jobs[tl.x];
   const int mt = tl.w & 3;
@@ -426,7 +431,7 @@ __global__ void __launch_bounds__(kGramThreads, BF ? 2 : 1) k_gram_tc(const CUte
   // BF16: 256 B rows [, 128 A rows], each split in place
   constexpr int RING = BF ? RING_BYTES / 2 : RING_BYTES;  // BF16: two CTAs per SM
   const int stage_bytes = BF ? (diag ? nbox * BM * RB : (BN + BM) * RB) : (diag ? 2 * B_BYTES : 2 * (B_BYTES + A_BYTES));
-  const int stages = min(MAXST, RING / stage_bytes);  // TF32: 3 (diagonal) or 2; BF16: 8
+  const int stages = min(MAXST, RING / stage_bytes);  // TF32: 3 (diagonal) or 2; BF16: 6, 3 or 2
   const int a_off = BF ? BN * RB : 2 * B_BYTES;              // A rows of an off-diagonal stage
   const uint32_t tx_bytes = (uint32_t)(nbox * BM * RB + (diag ? 0 : BM * RB));
   const uint32_t tcols = mt == 2 ? 2 * TMEM_COLS : TMEM_COLS;
@@ -437,8 +442,8 @@ __global__ void __launch_bounds__(kGramThreads, BF ? 2 : 1) k_gram_tc(const CUte
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(base + RING);
-  // bars[0..3): full (TMA landed), [3..6): split (heads and remainders
-  // written), [6..9): empty (MMAs done with the stage), [9]: done
+  // bars[0..MAXST): full (TMA landed), then split (heads and remainders
+  // written), then empty (MMAs done with the stage), [3 MAXST]: done
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 3 * MAXST + 1);
   volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -499,8 +504,8 @@ __global__ void __launch_bounds__(kGramThreads, BF ? 2 : 1) k_gram_tc(const CUte
       }
       unsigned char* sb = base + s * stage_bytes;
       if constexpr (BF) {
-        for (int q = 0; q < nbox; ++q) split_row_sw64(sb, t + q * BM);
-        if (!diag) split_row_sw64(sb + a_off, t);
+        if (t < nbox * BM) split_row(sb, t);
+        if (!diag && t < BM) split_row(sb + a_off, t);
       } else {
         split_block(sb, B_BYTES, nbox * A_BYTES / 16, t, SPLITTERS);
         if (!diag) split_block(sb + 2 * B_BYTES, A_BYTES, A_BYTES / 16, t, SPLITTERS);
@@ -529,15 +534,19 @@ __global__ void __launch_bounds__(kGramThreads, BF ? 2 : 1) k_gram_tc(const CUte
       }
       tc_fence_after();
       if constexpr (BF) {
-        // [head | remainder] rows: the remainders 32 bytes into each row
-        const uint32_t bh = su32(base + s * stage_bytes), bl = bh + 32;
+        // [head | remainder] rows: the remainders 64 bytes into each row
+        const uint32_t b0 = su32(base + s * stage_bytes);
         for (int q = 0; q < mt; ++q) {
           // diagonal: A sub-tile q is B rows [128 q, 128 q + 128)
-          const uint32_t ah = diag ? bh + (q0 + q) * BM * RB : bh + a_off, al = ah + 32;
+          const uint32_t a0 = diag ? b0 + (q0 + q) * BM * RB : b0 + a_off;
           const uint32_t d = tmem + (uint32_t)(q * TMEM_COLS);
-          mma<true>(d, sdesc<true>(ah), sdesc<true>(bh), id[q], kb > 0 ? 1u : 0u);
-          mma<true>(d, sdesc<true>(ah), sdesc<true>(bl), id[q], 1u);
-          mma<true>(d, sdesc<true>(al), sdesc<true>(bh), id[q], 1u);
+#pragma unroll
+          for (int k = 0; k < NSUB; ++k) {
+            const uint32_t ah = a0 + k * 32, al = ah + 64, bh = b0 + k * 32, bl = bh + 64;
+            mma<true>(d, sdesc(ah), sdesc(bh), id[q], (kb > 0 || k > 0) ? 1u : 0u);
+            mma<true>(d, sdesc(ah), sdesc(bl), id[q], 1u);
+            mma<true>(d, sdesc(al), sdesc(bh), id[q], 1u);
+          }
         }
       } else {
         const uint32_t bh = su32(base + s * stage_bytes), bl = bh + B_BYTES;
@@ -656,17 +665,14 @@ static PFN_cuTensorMapEncodeTiled_v12000 get_encode(std::string& err) {
 // Rank-2 FP32 tensor map over rows of `cols` elements (row stride ld
 // elements), box = one 128-byte k-block x 128 rows, 128-byte swizzle, zero
 // fill outside.
-// FP32 rows [rows x cols] with row stride ld (elements), boxes of 128 rows x
-// kblk values: kblk = 32 with the 128-byte swizzle (Gram, three-pass TF32
-// contraction), kblk = 16 with the 64-byte swizzle (BF16-mode contraction).
 static bool encode_rows(PFN_cuTensorMapEncodeTiled_v12000 encode, CUtensorMap* m, void* gaddr, int64_t cols, int64_t ld,
-                        int64_t rows, int kblk = KBLK_F32) {
+                        int64_t rows) {
   cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)ld * 4};
-  cuuint32_t box[2] = {(cuuint32_t)kblk, (cuuint32_t)BM};
+  cuuint32_t box[2] = {(cuuint32_t)KBLK, (cuuint32_t)BM};
   cuuint32_t estr[2] = {1, 1};
   return encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, gaddr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                kblk == KBLK_BF16 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                CU_TENSOR_MAP_SWIZZLE_128B,
                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -699,7 +705,6 @@ gnmppi_status tc_plan_create(const std::vector<InstDesc>& desc, void* dRW, const
   plan->bf16 = bf16;
   auto encode = get_encode(err);
   if (!encode) return GNMPPI_E_CUDA;
-  const int kblk = KBLK_F32;
   const int nb = (int)desc.size();
   if (bf16 && !W2) {
     err = "the BF16 contraction needs the split W copy";
@@ -713,7 +718,7 @@ gnmppi_status tc_plan_create(const std::vector<InstDesc>& desc, void* dRW, const
   int64_t part_elems = 0;
   for (int b = 0; b < nb; ++b) {
     const InstDesc& d = desc[b];
-    if (d.ldK % kblk != 0) {
+    if (d.ldK % KBLK != 0) {
       err = "sample padding is not a multiple of the k-block";
       return GNMPPI_E_ARG;
     }
@@ -723,13 +728,12 @@ gnmppi_status tc_plan_create(const std::vector<InstDesc>& desc, void* dRW, const
     }
     // contraction: one FP32 map over the instance's [dR; W] block
     if (!encode_rows(encode, &maps[b], reinterpret_cast<char*>(dRW) + 4 * (size_t)d.o_dR, d.ldK, d.ldK,
-                     d.nR + d.n, bf16 ? KBLK_BF16 : KBLK_F32)) {
+                     d.nR + d.n)) {
       err = "cuTensorMapEncodeTiled failed (contraction, instance " + std::to_string(b) + ")";
       return GNMPPI_E_CUDA;
     }
     // BF16 mode: the B rows come from the rollouts' split W copy
-    if (bf16 && !encode_rows(encode, &maps[3 * nb + b], const_cast<uint32_t*>(W2) + d.o_W2, d.ldK, d.ldK, d.n,
-                             KBLK_BF16)) {
+    if (bf16 && !encode_rows(encode, &maps[3 * nb + b], const_cast<uint32_t*>(W2) + d.o_W2, d.ldK, d.ldK, d.n)) {
       err = "cuTensorMapEncodeTiled failed (split W, instance " + std::to_string(b) + ")";
       return GNMPPI_E_CUDA;
     }
@@ -744,7 +748,7 @@ gnmppi_status tc_plan_create(const std::vector<InstDesc>& desc, void* dRW, const
     jc.b_row0 = bf16 ? d.nR : 0;
     jc.M = d.n;
     jc.Nc = d.nR + d.n;
-    jc.nkb = d.ldK / (bf16 ? KBLK_BF16 : KBLK_F32);
+    jc.nkb = d.ldK / KBLK;
     jc.x0 = 0;
     jc.out_off = d.o_P;
     jc.ldc = d.ldP;
@@ -767,9 +771,8 @@ gnmppi_status tc_plan_create(const std::vector<InstDesc>& desc, void* dRW, const
     }
     // Gram: FP32 maps over the P^T columns (nR) and the S columns (n) of [P^T | S]
     float* Pb = reinterpret_cast<float*>(P) + d.o_P;
-    const int gk = bf16 ? KBLK_BF16 : KBLK_F32;  // the BF16 mode's Gram: BF16 passes too
-    if (!encode_rows(encode, &maps[nb + b], Pb, d.nR, d.ldP, d.n, gk) ||
-        !encode_rows(encode, &maps[2 * nb + b], Pb + d.sP, d.n, d.ldP, d.n, gk)) {
+    if (!encode_rows(encode, &maps[nb + b], Pb, d.nR, d.ldP, d.n) ||
+        !encode_rows(encode, &maps[2 * nb + b], Pb + d.sP, d.n, d.ldP, d.n)) {
       err = "cuTensorMapEncodeTiled failed (Gram, instance " + std::to_string(b) + ")";
       return GNMPPI_E_CUDA;
     }
@@ -779,13 +782,13 @@ gnmppi_status tc_plan_create(const std::vector<InstDesc>& desc, void* dRW, const
     jg.map = nb + b;
     jg.M = d.n;
     jg.Nc = d.n;
-    jg.nkb = (d.nR + gk - 1) / gk;
+    jg.nkb = (d.nR + KBLK - 1) / KBLK;
     jg.out_off = d.o_nn;
     jg.ldc = d.n;
     jg.ccut = d.n;
     // nR beyond kGramChunkCols: one job per column chunk into the FP64 chunk
     // buffer, added up by k_gram_reduce
-    const int gchunk = kGramChunkCols / gk;
+    const int gchunk = kGramChunkCols / KBLK;
     const int nchunks = (jg.nkb + gchunk - 1) / gchunk;
     if (nchunks <= 1) {
       gram_tiles(nb + b, d.n, tg, bf16 != 0);
@@ -793,7 +796,7 @@ gnmppi_status tc_plan_create(const std::vector<InstDesc>& desc, void* dRW, const
       const int64_t nn = (int64_t)d.n * d.n;
       for (int c = 0; c < nchunks; ++c) {
         TcJob jc2 = jg;
-        jc2.x0 = c * gchunk * gk;
+        jc2.x0 = c * gchunk * KBLK;
         jc2.nkb = std::min(gchunk, jg.nkb - c * gchunk);
         jc2.out_sel = 2;
         jc2.out_off = part_elems + c * nn;
@@ -807,7 +810,7 @@ gnmppi_status tc_plan_create(const std::vector<InstDesc>& desc, void* dRW, const
     TcJob& js = jobs[2 * nb + b];
     js = jg;
     js.map = 2 * nb + b;
-    js.nkb = (d.n + gk - 1) / gk;
+    js.nkb = (d.n + KBLK - 1) / KBLK;
     js.out_sel = 1;
     if (d.lsq) gram_tiles(2 * nb + b, d.n, ts, bf16 != 0);
   }
@@ -843,6 +846,7 @@ gnmppi_status tc_plan_create(const std::vector<InstDesc>& desc, void* dRW, const
   plan->ntiles_c1 = (int)tc1.size();
   plan->ntiles_g = (int)tg.size();
   plan->nred = (int)red.size();
+  for (int b = 0; b < nb; ++b) plan->max_nkb = std::max(plan->max_nkb, jobs[b].nkb);
   bool ok = cudaMemcpyAsync(plan->d_maps, maps.data(), sizeof(CUtensorMap) * maps.size(), cudaMemcpyHostToDevice,
                             stream) == cudaSuccess;
   ok = ok && cudaMemcpyAsync(plan->d_jobs, jobs.data(), sizeof(TcJob) * jobs.size(), cudaMemcpyHostToDevice, stream) ==
@@ -883,14 +887,18 @@ gnmppi_status tc_plan_create(const std::vector<InstDesc>& desc, void* dRW, const
   return GNMPPI_OK;
 }
 
+int tc_contract_default_mt(const TcPlan& plan, int nsm) {
+  return 2 * plan.ntiles_c <= nsm || plan.max_nkb <= 8 ? 1 : 2;
+}
+
 cudaError_t tc_contract_launch(const TcPlan& plan, const InstState* d_st, float* P, cudaStream_t stream, int inject,
                                int mt) {
   if (plan.ntiles_c == 0) return cudaSuccess;
   if (plan.bf16 && mt == 1)
-    k_contract_tc<1><<<plan.ntiles_c1, kContractThreads, plan.smem1, stream>>>(plan.d_maps, plan.d_jobs, d_st,
+    k_contract_tc<1><<<plan.ntiles_c1, kContractThreads<1>, plan.smem1, stream>>>(plan.d_maps, plan.d_jobs, d_st,
                                                                                plan.d_tiles_c1, P, plan.d_err, inject);
   else if (plan.bf16)
-    k_contract_tc<2><<<plan.ntiles_c, kContractThreads, plan.smem, stream>>>(plan.d_maps, plan.d_jobs, d_st,
+    k_contract_tc<2><<<plan.ntiles_c, kContractThreads<2>, plan.smem, stream>>>(plan.d_maps, plan.d_jobs, d_st,
                                                                              plan.d_tiles_c, P, plan.d_err, inject);
   else
     k_gram_tc<true><<<plan.ntiles_c, kGramThreads, plan.smem, stream>>>(plan.d_maps, plan.d_jobs, d_st,

@@ -51,6 +51,7 @@ struct TcPlan {
   int4* d_tiles_g = nullptr;      // (job, first row, first column, sub-tiles | 4 diagonal) of the Gram products
   int ntiles_c = 0, ntiles_c1 = 0, ntiles_g = 0;
   int smem = 0, smem1 = 0;
+  int max_nkb = 0;                // most k-blocks of a contraction tile
   int bf16 = 1;
   float* d_part = nullptr;        // FP32 chunk results of the chunked Grams
   GramRed* d_red = nullptr;       // one record per chunked instance
@@ -73,6 +74,13 @@ gnmppi_status tc_plan_create(const std::vector<InstDesc>& desc, void* dRW, const
 // mt (BF16 mode): A sub-tiles per CTA, 2 (one CTA per SM) or 1 (two per SM).
 cudaError_t tc_contract_launch(const TcPlan& plan, const InstState* d_st, float* P, cudaStream_t stream, int inject,
                                int mt);
+
+// mt without tuning: 1 where 256-row tiles would leave half the nsm SMs without
+// one, or where a tile is so short (K' <= 256) that starting up and storing it
+// weigh as much as its k-blocks; else 2.  mt = 2 against 1 (us): one chain of M =
+// 10 39 / 33, eight 41 / 35, 64 174 / 178; 256 at K' = 1024 657 / 657, at K' = 256
+// 278 / 252; 16 of M = 32 at K' = 2048 729 / 780.
+int tc_contract_default_mt(const TcPlan& plan, int nsm);
 
 // A = P^T P and, for instances in LSQ mode, S2 = S S^T (FP64 outputs) from
 // three passes over [P^T | S] split in shared memory (BF16 head + remainder

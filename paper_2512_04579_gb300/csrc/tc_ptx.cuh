@@ -66,15 +66,13 @@ __device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* map, u
 
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of
 // 128 bytes, 8-row groups 1024 bytes apart (SBO), descriptor version 1.
-// ROW64: 64-byte swizzle, rows of 64 bytes, 8-row groups 512 bytes apart.
-template <bool ROW64 = false>
 __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
   uint64_t d = 0;
   d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
   d |= (uint64_t)1 << 16;
-  d |= (uint64_t)((ROW64 ? 512 : 1024) >> 4) << 32;
+  d |= (uint64_t)(1024 >> 4) << 32;
   d |= (uint64_t)1 << 46;
-  d |= (uint64_t)(ROW64 ? 4 : 2) << 61;
+  d |= (uint64_t)2 << 61;
   return d;
 }
 
