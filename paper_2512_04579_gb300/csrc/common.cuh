@@ -383,6 +383,22 @@ struct Chain {
   }
 };
 
+// 1 / sqrt(q) of a link's squared length.  FAST is the hardware approximation
+// alone; rsqrtf adds three instructions per link that rescale a subnormal q, and
+// is bitwise the same for every other q.  For a subnormal q (a link shorter
+// than 1.1e-19) FAST gives infinity, which no later step takes back: it makes
+// the rollout's cost infinite or NaN.  So the sample kernels roll out with FAST
+// and run the rare warp that ends with a non-finite cost again without it
+// (samples phase of 256 chains, M = 10, N = 100, K = 2048: 2.01 -> 1.85 ms; 16 of
+// M = 32, N = 200, K = 4096: 2.32 -> 2.16; 64 of M = 16: 1.01 -> 0.92).
+template <bool FAST>
+__device__ __forceinline__ float link_rsqrt(float q) {
+  if constexpr (!FAST) return rsqrtf(q);
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(q));
+  return r;
+}
+
 // FP32 chain on paired FP32 instructions: a mass's position, velocity and
 // acceleration are float2, updated with FFMA2 / FADD2 / FMUL2 (sm_100+); 1/m
 // is folded into the spring, damping and control constants.  The state array
@@ -415,6 +431,7 @@ struct Chain<float, F> {
     pref = nullptr;
   }
   // acc = (-c v + link forces + u on the last mass) / m - g y
+  template <bool FAST>
   __device__ __forceinline__ void accel(const float2* p, const float2* v, float2 um, float2* acc) const {
 #pragma unroll
     for (int i = 0; i < F; ++i) acc[i] = __ffma2_rn(v[i], cneg, grav);
@@ -423,7 +440,7 @@ struct Chain<float, F> {
     for (int i = 0; i < F; ++i) {
       const float2 d = (i == 0) ? p[0] : __ffma2_rn(p[i - 1], mneg1, p[i]);
       const float q = fmaf(d.x, d.x, d.y * d.y);
-      const float rinv = rsqrtf(q);
+      const float rinv = link_rsqrt<FAST>(q);
       const float dd = fmaf(q, rinv, -l0);
       const float t = fmaf(k3m * dd, dd, km) * dd;
       const float fr = t * rinv;  // (k d + k3 d^3) / (m |d|): the link pulls mass i back, mass i-1 on
@@ -431,12 +448,14 @@ struct Chain<float, F> {
       if (i > 0) acc[i - 1] = __ffma2_rn(make_float2(fr, fr), d, acc[i - 1]);
     }
   }
-  __device__ __forceinline__ void step(float* xs, const float* u) const {
+  __device__ __forceinline__ void step(float* xs, const float* u) const { step_t<false>(xs, u); }
+  template <bool FAST>
+  __device__ __forceinline__ void step_t(float* xs, const float* u) const {
     float2* p = reinterpret_cast<float2*>(xs);
     float2* v = p + F;
     const float2 um = make_float2(u[0] * mass_inv, u[1] * mass_inv);
     float2 ap[F], av[F], tp[F], tv[F], acc[F];
-    accel(p, v, um, acc);
+    accel<FAST>(p, v, um, acc);
 #pragma unroll
     for (int i = 0; i < F; ++i) {
       ap[i] = v[i];
@@ -444,7 +463,7 @@ struct Chain<float, F> {
       tp[i] = __ffma2_rn(hh2, v[i], p[i]);
       tv[i] = __ffma2_rn(hh2, acc[i], v[i]);
     }
-    accel(tp, tv, um, acc);
+    accel<FAST>(tp, tv, um, acc);
 #pragma unroll
     for (int i = 0; i < F; ++i) {
       ap[i] = __ffma2_rn(two, tv[i], ap[i]);
@@ -452,7 +471,7 @@ struct Chain<float, F> {
       tp[i] = __ffma2_rn(hh2, tv[i], p[i]);
       tv[i] = __ffma2_rn(hh2, acc[i], v[i]);
     }
-    accel(tp, tv, um, acc);
+    accel<FAST>(tp, tv, um, acc);
 #pragma unroll
     for (int i = 0; i < F; ++i) {
       ap[i] = __ffma2_rn(two, tv[i], ap[i]);
@@ -460,7 +479,7 @@ struct Chain<float, F> {
       tp[i] = __ffma2_rn(hh, tv[i], p[i]);
       tv[i] = __ffma2_rn(hh, acc[i], v[i]);
     }
-    accel(tp, tv, um, acc);
+    accel<FAST>(tp, tv, um, acc);
 #pragma unroll
     for (int i = 0; i < F; ++i) {
       p[i] = __ffma2_rn(hh6, __fadd2_rn(ap[i], tv[i]), p[i]);

@@ -146,27 +146,30 @@ static __global__ void __launch_bounds__(128) k_noise_f64(RollArgs a) {
   if (j + 1 < I.n && GNM_IN(j + 1, I.n)) W[I.ldK] = s[1] * z1;
 }
 
-template <class Model, typename T, typename S, bool ANTI>
-__global__ void __launch_bounds__(128) k_samples(RollArgs a) {
-  constexpr int NX = Model::NX, NU = Model::NU;
-  const int2 bm = a.bmap[blockIdx.x];
-  const InstDesc I = a.inst[bm.x];
-  if (a.st[bm.x].status != 0) return;
-  // shared: U, s (n each), the nominal residual r (nR) and the reference, in T
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* sU = reinterpret_cast<T*>(smem_raw);
-  T* sS = sU + I.n;
-  T* sR = sS + I.n;
-  T* sRef = sR + I.nR;
-  const T* rg = reinterpret_cast<const T*>(a.r) + I.o_R;
-  for (int j = threadIdx.x; j < I.n; j += blockDim.x) {
-    sU[j] = (T)a.U[I.o_U + j];
-    sS[j] = (T)a.s[I.o_U + j];
-  }
-  for (int j = threadIdx.x; j < I.nR; j += blockDim.x) sR[j] = rg[j];
-  for (int j = threadIdx.x; j < RefSize<Model>::value; j += blockDim.x) sRef[j] = (T)a.xref[I.o_xref + j];
-  __syncthreads();
+// A model's step; the FP32 chain's with FAST reciprocal square roots (link_rsqrt).
+template <bool FAST, class Model, typename T>
+__device__ __forceinline__ void model_step(const Model& md, T* x, const T* u) {
+  md.step(x, u);
+}
+template <bool FAST, int F>
+__device__ __forceinline__ void model_step(const Chain<float, F>& md, float* x, const float* u) {
+  md.template step_t<FAST>(x, u);
+}
+template <class Model>
+struct HasFast {
+  static constexpr bool value = false;
+};
+template <int F>
+struct HasFast<Chain<float, F>> {
+  static constexpr bool value = true;
+};
 
+// One rollout of k_samples from the staged arrays, outputs included; false if
+// its sample or pair is dropped.
+template <class Model, typename T, typename S, bool ANTI, bool FAST>
+__device__ __forceinline__ bool sample_rollout(const RollArgs& a, const InstDesc& I, int2 bm, const T* sU, const T* sS,
+                                               const T* sR, const T* sRef) {
+  constexpr int NX = Model::NX, NU = Model::NU;
   const int per_block = ANTI ? kPairsPerBlock : kSamplesPerBlock;
   const int local = ANTI ? (threadIdx.x >> 1) : threadIdx.x;
   const int m = bm.y * per_block + local;
@@ -265,7 +268,7 @@ __global__ void __launch_bounds__(128) k_samples(RollArgs a) {
     {
       T ua[Model::NU];
       dead_zone<T, Model::NU>(u, ua, uf_t);
-      md.step(x, ua);
+      model_step<FAST>(md, x, ua);
     }
   }
   em.col = dR + I.N * stage_stride;
@@ -294,6 +297,33 @@ __global__ void __launch_bounds__(128) k_samples(RollArgs a) {
       for (int row = par; row < rows; row += (ANTI ? 2 : 1)) put(dR + (int64_t)row * I.ldK + m, (T)0);
       for (int j = par; j < I.n; j += (ANTI ? 2 : 1)) put_w(Wm, W2b, I.ldK, j, m, (T)0);
     }
+  }
+  return ok;
+}
+
+template <class Model, typename T, typename S, bool ANTI>
+__global__ void __launch_bounds__(128) k_samples(RollArgs a) {
+  const int2 bm = a.bmap[blockIdx.x];
+  const InstDesc I = a.inst[bm.x];
+  if (a.st[bm.x].status != 0) return;
+  // shared: U, s (n each), the nominal residual r (nR) and the reference, in T
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* sU = reinterpret_cast<T*>(smem_raw);
+  T* sS = sU + I.n;
+  T* sR = sS + I.n;
+  T* sRef = sR + I.nR;
+  const T* rg = reinterpret_cast<const T*>(a.r) + I.o_R;
+  for (int j = threadIdx.x; j < I.n; j += blockDim.x) {
+    sU[j] = (T)a.U[I.o_U + j];
+    sS[j] = (T)a.s[I.o_U + j];
+  }
+  for (int j = threadIdx.x; j < I.nR; j += blockDim.x) sR[j] = rg[j];
+  for (int j = threadIdx.x; j < RefSize<Model>::value; j += blockDim.x) sRef[j] = (T)a.xref[I.o_xref + j];
+  __syncthreads();
+  const bool ok = sample_rollout<Model, T, S, ANTI, true>(a, I, bm, sU, sS, sR, sRef);
+  if constexpr (HasFast<Model>::value) {
+    if (__any_sync(0xffffffffu, !ok))  // a subnormal link length, or a diverged rollout
+      sample_rollout<Model, T, S, ANTI, false>(a, I, bm, sU, sS, sR, sRef);
   }
 }
 

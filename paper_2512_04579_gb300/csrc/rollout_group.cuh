@@ -199,6 +199,7 @@ struct ChainGroup<float, FL, G, FX> {
       }
     }
   }
+  template <bool FAST>
   __device__ __forceinline__ void accel(const float2* p, const float2* v, float2 um, float2* acc) const {
     float2 prev;
     prev.x = __shfl_up_sync(mask, p[FL - 1].x, 1, G);
@@ -213,7 +214,7 @@ struct ChainGroup<float, FL, G, FX> {
       d[j] = __fadd2_rn(__ffma2_rn((j == 0) ? prev : p[j - 1], mneg1, p[j]), dref[j]);
       const bool real = this->real(j);
       const float q = real ? fmaf(d[j].x, d[j].x, d[j].y * d[j].y) : 1.f;
-      const float rinv = rsqrtf(q);
+      const float rinv = link_rsqrt<FAST>(q);
       const float dd = fmaf(q, rinv, -l0);
       fr[j] = real ? fmaf(k3m * dd, dd, km) * dd * rinv : 0.f;
     }
@@ -233,12 +234,14 @@ struct ChainGroup<float, FL, G, FX> {
       acc[j] = real(j) ? a : make_float2(0.f, 0.f);
     }
   }
-  __device__ __forceinline__ void step(float* xs, const float* u) const {
+  __device__ __forceinline__ void step(float* xs, const float* u) const { step_t<false>(xs, u); }
+  template <bool FAST>
+  __device__ __forceinline__ void step_t(float* xs, const float* u) const {
     float2* p = reinterpret_cast<float2*>(xs);
     float2* v = p + FL;
     const float2 um = make_float2(u[0] * mass_inv, u[1] * mass_inv);
     float2 ap[FL], av[FL], tp[FL], tv[FL], acc[FL];
-    accel(p, v, um, acc);
+    accel<FAST>(p, v, um, acc);
 #pragma unroll
     for (int i = 0; i < FL; ++i) {
       ap[i] = v[i];
@@ -246,7 +249,7 @@ struct ChainGroup<float, FL, G, FX> {
       tp[i] = __ffma2_rn(hh2, v[i], p[i]);
       tv[i] = __ffma2_rn(hh2, acc[i], v[i]);
     }
-    accel(tp, tv, um, acc);
+    accel<FAST>(tp, tv, um, acc);
 #pragma unroll
     for (int i = 0; i < FL; ++i) {
       ap[i] = __ffma2_rn(two, tv[i], ap[i]);
@@ -254,7 +257,7 @@ struct ChainGroup<float, FL, G, FX> {
       tp[i] = __ffma2_rn(hh2, tv[i], p[i]);
       tv[i] = __ffma2_rn(hh2, acc[i], v[i]);
     }
-    accel(tp, tv, um, acc);
+    accel<FAST>(tp, tv, um, acc);
 #pragma unroll
     for (int i = 0; i < FL; ++i) {
       ap[i] = __ffma2_rn(two, tv[i], ap[i]);
@@ -262,7 +265,7 @@ struct ChainGroup<float, FL, G, FX> {
       tp[i] = __ffma2_rn(hh, tv[i], p[i]);
       tv[i] = __ffma2_rn(hh, acc[i], v[i]);
     }
-    accel(tp, tv, um, acc);
+    accel<FAST>(tp, tv, um, acc);
 #pragma unroll
     for (int i = 0; i < FL; ++i) {
       p[i] = __ffma2_rn(hh6, __fadd2_rn(ap[i], tv[i]), p[i]);
@@ -291,48 +294,20 @@ __device__ __forceinline__ T group_sum(T v, int G, unsigned mask) {
   return v;
 }
 
-// k_samples for groups.  Every lane of a group emits its rows in the same
-// order and the partner group emits the same rows, so the difference is taken
-// row by row with one xor-shuffle per emitted row.
-template <typename T, typename S, int FL, int G, int FX = 0>
-__global__ void __launch_bounds__(256, 2) k_samples_group(RollArgs a) {
-  constexpr int PAIRS = 256 / (2 * G);
-  const int2 bm = a.bmap[blockIdx.x];
-  const InstDesc I = a.inst[bm.x];
-  if (a.st[bm.x].status != 0) return;
-  // Shared: U, s (n each), then the nominal residual and the target positions
-  // in a group-interleaved layout, so that the 2G lanes of a pair read 2G
-  // consecutive words (lane lg's mass slot j at [2G j + 2 lg], the controls
-  // after the SL mass slots of a stage):
-  //   sR[k RS + 2G j + 2 lg + c] = r[k rps + 2 (lg FL + j) + c],
-  //   sR[k RS + 2 SL + c]        = r[k rps + 2F + c],   sRef likewise, zero-padded.
-  constexpr int SL = G * FL;      // mass slots of a rollout group
-  constexpr int RS = 2 * SL + 2;  // interleaved words per stage
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* sU = reinterpret_cast<T*>(smem_raw);
-  T* sS = sU + I.n;
-  T* sR = sS + I.n;
-  T* sRef = sR + (int64_t)(I.N + 1) * RS;
-  const T* rg = reinterpret_cast<const T*>(a.r) + I.o_R;
-  const int rps = 2 * I.F + 2;
-  for (int j = threadIdx.x; j < I.n; j += blockDim.x) {
-    sU[j] = (T)a.U[I.o_U + j];
-    sS[j] = (T)a.s[I.o_U + j];
-  }
-  for (int idx = threadIdx.x; idx < I.nR; idx += blockDim.x) {
-    const int k = idx / rps, i = idx - k * rps, q = i >> 1;
-    const int w = i < 2 * I.F ? (q % FL) * 2 * G + 2 * (q / FL) + (i & 1) : 2 * SL + (i - 2 * I.F);
-    sR[k * RS + w] = rg[idx];
-  }
-  // targets (FP32 model: their offsets from the initial positions)
-  constexpr bool REL = ChainGroup<T, FL, G, FX>::kRelative;
-  for (int idx = threadIdx.x; idx < 2 * SL; idx += blockDim.x) {
-    const int q = idx >> 1;
-    sRef[(q % FL) * 2 * G + 2 * (q / FL) + (idx & 1)] =
-        q < I.F ? (T)(a.xref[I.o_xref + idx] - (REL ? a.x0[I.o_x0 + idx] : 0.0)) : (T)0;
-  }
-  __syncthreads();
+template <bool FAST, typename T, int FL, int G, int FX>
+__device__ __forceinline__ void group_step(const ChainGroup<T, FL, G, FX>& md, T* x, const T* u) {
+  if constexpr (sizeof(T) == 4) md.template step_t<FAST>(x, u);
+  else md.step(x, u);
+}
 
+// One rollout of k_samples_group from the staged arrays, outputs included;
+// false if its pair is dropped.
+template <typename T, typename S, int FL, int G, int FX, bool FAST>
+__device__ __forceinline__ bool group_rollout(const RollArgs& a, const InstDesc& I, int2 bm, const T* sU, const T* sS,
+                                              const T* sR, const T* sRef) {
+  constexpr int PAIRS = 256 / (2 * G), SL = G * FL, RS = 2 * SL + 2;
+  constexpr bool REL = ChainGroup<T, FL, G, FX>::kRelative;
+  const int rps = 2 * I.F + 2;
   const int lane = threadIdx.x & 31;
   const int lg = lane & (G - 1);
   const bool plus = (lane & G) == 0;
@@ -420,7 +395,7 @@ __global__ void __launch_bounds__(256, 2) k_samples_group(RollArgs a) {
     {
       T ua[2];
       dead_zone<T, 2>(u, ua, uf_t);
-      md.step(x, ua);
+      group_step<FAST>(md, x, ua);
     }
   }
   em.base = I.N * rps;
@@ -449,6 +424,53 @@ __global__ void __launch_bounds__(256, 2) k_samples_group(RollArgs a) {
     for (int row = lg; row < rows; row += G) put(dR + (int64_t)row * I.ldK + m, (T)0);
     for (int j = lg; j < I.n; j += G) put_w(Wm, W2b, I.ldK, j, m, (T)0);
   }
+  return ok;
+}
+
+// k_samples for groups.  Every lane of a group emits its rows in the same
+// order and the partner group emits the same rows, so the difference is taken
+// row by row with one xor-shuffle per emitted row.
+template <typename T, typename S, int FL, int G, int FX = 0>
+__global__ void __launch_bounds__(256, 2) k_samples_group(RollArgs a) {
+  const int2 bm = a.bmap[blockIdx.x];
+  const InstDesc I = a.inst[bm.x];
+  if (a.st[bm.x].status != 0) return;
+  // Shared: U, s (n each), then the nominal residual and the target positions
+  // in a group-interleaved layout, so that the 2G lanes of a pair read 2G
+  // consecutive words (lane lg's mass slot j at [2G j + 2 lg], the controls
+  // after the SL mass slots of a stage):
+  //   sR[k RS + 2G j + 2 lg + c] = r[k rps + 2 (lg FL + j) + c],
+  //   sR[k RS + 2 SL + c]        = r[k rps + 2F + c],   sRef likewise, zero-padded.
+  constexpr int SL = G * FL;      // mass slots of a rollout group
+  constexpr int RS = 2 * SL + 2;  // interleaved words per stage
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* sU = reinterpret_cast<T*>(smem_raw);
+  T* sS = sU + I.n;
+  T* sR = sS + I.n;
+  T* sRef = sR + (int64_t)(I.N + 1) * RS;
+  const T* rg = reinterpret_cast<const T*>(a.r) + I.o_R;
+  const int rps = 2 * I.F + 2;
+  for (int j = threadIdx.x; j < I.n; j += blockDim.x) {
+    sU[j] = (T)a.U[I.o_U + j];
+    sS[j] = (T)a.s[I.o_U + j];
+  }
+  for (int idx = threadIdx.x; idx < I.nR; idx += blockDim.x) {
+    const int k = idx / rps, i = idx - k * rps, q = i >> 1;
+    const int w = i < 2 * I.F ? (q % FL) * 2 * G + 2 * (q / FL) + (i & 1) : 2 * SL + (i - 2 * I.F);
+    sR[k * RS + w] = rg[idx];
+  }
+  // targets (FP32 model: their offsets from the initial positions)
+  constexpr bool REL = ChainGroup<T, FL, G, FX>::kRelative;
+  for (int idx = threadIdx.x; idx < 2 * SL; idx += blockDim.x) {
+    const int q = idx >> 1;
+    sRef[(q % FL) * 2 * G + 2 * (q / FL) + (idx & 1)] =
+        q < I.F ? (T)(a.xref[I.o_xref + idx] - (REL ? a.x0[I.o_x0 + idx] : 0.0)) : (T)0;
+  }
+  __syncthreads();
+
+  const bool ok = group_rollout<T, S, FL, G, FX, true>(a, I, bm, sU, sS, sR, sRef);
+  if (sizeof(T) == 4 && __any_sync(0xffffffffu, !ok))  // a subnormal link length, or a diverged rollout
+    group_rollout<T, S, FL, G, FX, false>(a, I, bm, sU, sS, sR, sRef);
 }
 
 // Line search / nominal / FP64 cost for groups: one group per (instance, candidate).
