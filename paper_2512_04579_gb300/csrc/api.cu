@@ -953,7 +953,7 @@ static gnmppi_status launch_iteration_t(gnmppi_t h, uint32_t it, int shrink, cud
   }
   MARK(7);
   if (ON(7)) {
-    k_update<T><<<h->batch, 128, 0, h->stream>>>(sa);
+    k_update<T><<<h->batch, 512, 0, h->stream>>>(sa);
     CKL();
     h->launches++;
   }

@@ -764,11 +764,13 @@ __global__ void __launch_bounds__(256) k_mppi_step(SolveArgs a) {
   }
 }
 
-// One CTA (128 threads) per instance: line-search argmin (ties to the smallest
+// One CTA (512 threads: the copy of the chosen candidate's residual, nR values,
+// is all latency; with 128 it took 59 us at nR = 25726, 20 now, 14 and 10 at
+// 2018) per instance: line-search argmin (ties to the smallest
 // j; alpha = 0 last when monotone), U += alpha* delta, r <- R(U + alpha* delta),
 // and, in Algorithm-1 solves, s <- sqrt(beta) s.
 template <typename T>
-__global__ void __launch_bounds__(128) k_update(SolveArgs a) {
+__global__ void __launch_bounds__(512) k_update(SolveArgs a) {
   const int b = blockIdx.x;
   InstState& st = a.st[b];
   if (st.status != 0) return;
@@ -806,8 +808,9 @@ __global__ void __launch_bounds__(128) k_update(SolveArgs a) {
     if (a.shrink) a.s[I.o_U + i] *= a.cs.beta_sqrt;
   }
   if (js < a.cs.L) {
-    T* r = reinterpret_cast<T*>(a.r) + I.o_R;
-    const T* src = reinterpret_cast<const T*>(a.RL) + I.o_RL + (int64_t)js * I.nR;
+    T* __restrict__ r = reinterpret_cast<T*>(a.r) + I.o_R;
+    const T* __restrict__ src = reinterpret_cast<const T*>(a.RL) + I.o_RL + (int64_t)js * I.nR;
+#pragma unroll 8
     for (int i = threadIdx.x; i < I.nR; i += blockDim.x) r[i] = src[i];
   }
   if (threadIdx.x == 0) {

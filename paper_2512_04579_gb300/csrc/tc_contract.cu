@@ -20,7 +20,7 @@
 //                       [head | remainder] row (each thread one row),
 //        warp 1 lane 0  issues tcgen05.mma (M=128, N = the W rows, K=16) per
 //                       sub-tile,
-//        warps 0-3      read TMEM back (tcgen05.ld 32x32b, one lane per
+//        warps 0-7      read TMEM back (tcgen05.ld 32x32b, one lane per
 //                       [P^T | S] column) and store 32 consecutive columns
 //                       per warp store (the S columns from column sP on);
 //    FP32 mode: the three-pass TF32 kernel of (2) on the FP32 [dR; W] block.
@@ -117,7 +117,7 @@ __device__ __forceinline__ void split_row(unsigned char* p, int row) {
 // BF16 MMAs of K = 16 (head x head, head x remainder, remainder x head, the
 // remainders 64 bytes into the rows), which keeps FP32-level accuracy (the
 // dropped remainder x remainder term is ~2^-18 relative).  Warp 0 lane 0 TMA,
-// warp 1 lane 0 MMA, warps 2 on split; warps 0-3 read TMEM back.
+// warp 1 lane 0 MMA, warps 2 on split; warps 0-7 (MT = 1: 0-3) read TMEM back.
 //
 // What bounds a tile is shared memory's 128 bytes per clock: per k-block the
 // TMA fill (64 KB), the A rows' split (32 + 32 KB) and the MMAs' operand reads
@@ -125,7 +125,8 @@ __device__ __forceinline__ void split_row(unsigned char* p, int row) {
 // values (64-byte rows) took 1450 each: half-width TMA rows and twice the
 // barriers (256 chains of M = 10, K = 2048: 0.72 ms, 0.66 now; one: 47 us, 39
 // now; DRAM's floor at 256 is 0.44 ms).  Four splitter warps with two rows per
-// thread took as long as eight.
+// thread took as long as eight; the epilogue on eight warps instead of four took
+// 0.66 ms to 0.64.
 //
 // MT: A sub-tiles per CTA.  MT = 2: 256 A rows, a 3-stage ring of 64 KB, one
 // CTA per SM; MT = 1: 128 A rows, a 2-stage ring of 48 KB, two CTAs per SM, one
@@ -271,26 +272,29 @@ __global__ void __launch_bounds__(kContractThreads<MT>, 3 - MT) k_contract_tc(co
   __syncwarp();
 
   // ---------------- epilogue: TMEM -> registers -> rows of [P^T | S]
-  // Lane l of warp w holds A row i = row_org + 128 sub + 32 w + l, i.e.
+  // Lane l of warp w holds A row i = row_org + 128 sub + 32 (w mod 4) + l, i.e.
   // output column i; a 32-column TMEM load gives it 32 consecutive output
-  // rows j, and each store of the warp covers 32 consecutive columns.
+  // rows j, and each store of the warp covers 32 consecutive columns.  MT = 2:
+  // warps 0-7, two per 32 lanes, each every other 32 rows.
+  constexpr int EW = MT == 2 ? 2 : 1;
   const bool ok = mbar_wait(done, 0, abort, false);
   tc_fence_after();
   // tcgen05.ld is warp-collective: the whole warp takes the same branch
-  if (warp >= 4) {
-    // no TMEM lanes of their own
+  if (warp >= 4 * EW) {
+    // no rows of their own
   } else if (__all_sync(0xffffffffu, ok && !*abort)) {
+    const int quad = warp & 3;
     float* out = D + J.out_off;
     const int jn = min(BN, J.M - tl.z * BN);  // output rows of this tile
 #pragma unroll 1
     for (int sub = 0; sub < mt; ++sub) {
-      const int i = row_org + sub * BM + warp * 32 + lane;
+      const int i = row_org + sub * BM + quad * 32 + lane;
       const bool live = i < J.Nc;
       const int colw = i < J.ccut ? i : i + J.cgap;
 #pragma unroll 1
-      for (int c = 0; c * 32 < jn; ++c) {  // uniform over the warp
+      for (int c = warp >> 2; c * 32 < jn; c += EW) {  // uniform over the warp
         uint32_t v[32];
-        tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(sub * TMEM_COLS + c * 32), v);
+        tmem_ld32(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(sub * TMEM_COLS + c * 32), v);
         const int j0 = tl.z * BN + c * 32;
         if (live) {
 #pragma unroll
@@ -325,16 +329,18 @@ __device__ __forceinline__ float tf32_head(float x) {
 // epilogue).  IEEE 754 binary32 -> binary64: the sign stays, a normal
 // exponent is rebiased by 1023 - 127 = 896, the 23 fraction bits become the
 // top of the 52 (the low 3 of them land in the low word's top 3 bits);
-// zeros, infinities and NaNs keep their class; subnormals (rare here) take
-// the hardware conversion.
+// zeros, infinities and NaNs keep their class.  No branches, so that a
+// chunk's conversions overlap; subnormals (rare here) are the caller's.
+__device__ __forceinline__ bool subnormal_f32(uint32_t u) { return (u & 0x7FFFFFFFu) - 1u < 0x007FFFFFu; }
+__device__ __forceinline__ double widen_normal_f32(uint32_t u) {
+  const uint32_t a = u & 0x7FFFFFFFu;
+  uint32_t hi = (a >> 3) + (896u << 20);
+  hi = a >= 0x7F800000u ? 0x7FF00000u | ((a & 0x007FFFFFu) >> 3) : hi;
+  hi = a == 0u ? 0u : hi;
+  return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
+}
 __device__ __forceinline__ double widen_f32(uint32_t u) {
-  const uint32_t a = u & 0x7FFFFFFFu, sgn = u & 0x80000000u;
-  uint32_t hi;
-  if (a >= 0x7F800000u) hi = sgn | 0x7FF00000u | ((a & 0x007FFFFFu) >> 3);
-  else if (a >= 0x00800000u) hi = sgn | ((a >> 3) + (896u << 20));
-  else if (a == 0u) hi = sgn;
-  else return (double)__uint_as_float(u);
-  return __hiloint2double((int)hi, (int)(u << 29));
+  return subnormal_f32(u) ? (double)__uint_as_float(u) : widen_normal_f32(u);
 }
 
 // Splits `n4` float4 of a landed operand block in place: head (TF32) at p,
@@ -368,21 +374,20 @@ __device__ __forceinline__ void store_block(T* out, const T* stg, const TcJob& J
   const int col = cbase + lane;
   if (col < J.Nc) {
     const int colw = col < J.ccut ? col : col + J.cgap;
-#pragma unroll 4
+    T* o = out + (int64_t)row0 * J.ldc + colw;
+    const int rows = min(32, J.M - row0);
+#pragma unroll 8
     for (int rr = 0; rr < 32; ++rr)
-      if (row0 + rr < J.M && GNM_IN((int64_t)(row0 + rr) * J.ldc + colw, (int64_t)J.M * J.ldc))
-        out[(int64_t)(row0 + rr) * J.ldc + colw] = stg[rr * 33 + lane];
+      if (rr < rows && GNM_IN((int64_t)(row0 + rr) * J.ldc + colw, (int64_t)J.M * J.ldc))
+        o[(int64_t)rr * J.ldc] = stg[rr * 33 + lane];
   }
-  if (mirror) {
-    const int rowt = row0 + lane;
-    if (rowt < J.M) {
-#pragma unroll 4
-      for (int rr = 0; rr < 32; ++rr) {
-        const int colt = cbase + rr;
-        if (colt < J.Nc && GNM_IN((int64_t)colt * J.ldc + rowt, (int64_t)J.M * J.ldc))
-          out[(int64_t)colt * J.ldc + rowt] = stg[lane * 33 + rr];
-      }
-    }
+  if (mirror && row0 + lane < J.M) {
+    T* o = out + (int64_t)cbase * J.ldc + row0 + lane;
+    const int cols = min(32, J.Nc - cbase);
+#pragma unroll 8
+    for (int rr = 0; rr < 32; ++rr)
+      if (rr < cols && GNM_IN((int64_t)(cbase + rr) * J.ldc + row0 + lane, (int64_t)J.M * J.ldc))
+        o[(int64_t)rr * J.ldc] = stg[lane * 33 + rr];
   }
 }
 
@@ -390,7 +395,7 @@ __device__ __forceinline__ void store_block(T* out, const T* stg, const TcJob& J
 // tl.w = sub-tiles (1 or 2) | 4 if the tile sits on the diagonal.  Per stage
 // (one 32-column k-block): B head and remainder (256 rows), and for an
 // off-diagonal tile A head and remainder (128 rows).  Warp 0 lane 0 TMA, warp
-// 1 lane 0 MMA, warps 2-9 split; warps 0-3 read TMEM back.
+// 1 lane 0 MMA, warps 2-9 split; warps 0-7 read TMEM back.
 // CONTRACT: the same three-pass product for the FP32 mode's contraction
 // [P^T | S] = W^T [dR | W] (off-diagonal tiles only, A rows a_row0 + i and B
 // rows b_row0 + j of the instance's FP32 [dR; W] map), FP32 output into out0
@@ -404,20 +409,26 @@ constexpr int kGramThreads = 64 + 2 * BM;
 // diagonal tile with two sub-tiles runs as two CTAs (tl.w bit 3 marks the
 // second), the first loading only the 128 B rows its MMAs read.  Same
 // products in the same order per output as one CTA per diagonal tile
-// (0.266 -> 0.215 ms per launch at 256 instances of n = 200).  k-blocks of 16
-// values took 90 us for one chain of M = 10, 74 now, and as long for 256.
+// (0.266 -> 0.215 ms per launch at 256 instances of n = 200).  Where such tiles
+// number no more than the SMs (a few instances), each has an SM to itself and
+// takes a 192 KB ring (up to 12 stages), and the FP32 mode's diagonal tiles
+// run as two CTAs too.  The epilogue was a third of a tile's time (one chain: 19
+// of 59 us, four warps and a branch per widened entry): eight warps and
+// branch-free widening took the BF16 mode's Gram of one chain of M = 10 from 74
+// to 53 us, of 256 from 215 to 174; with the split tiles the FP32 mode's from
+// 115 to 68 and from 297 to 221.
 template <bool CONTRACT, bool BF = false>
 __global__ void __launch_bounds__(kGramThreads, BF ? 2 : 1) k_gram_tc(const CUtensorMap* __restrict__ maps, const TcJob* __restrict__ jobs,
                                                     const InstState* __restrict__ st, const int4* __restrict__ tiles,
                                                     void* __restrict__ out0, double* __restrict__ S2,
                                                     float* __restrict__ part,
-                                                    int* __restrict__ err, int inject) {
+                                                    int* __restrict__ err, int inject, int ring) {
   using TO = typename std::conditional<CONTRACT, float, double>::type;
   static_assert(!(CONTRACT && BF), "the BF16 contraction is k_contract_tc");
   constexpr int NSUB = BF ? 2 : 4;  // MMAs (TF32 K = 8, BF16 K = 16) per k-block
   constexpr int RB = ROW_BYTES;  // bytes of one landed row of a k-block
   constexpr int SPLITTERS = kGramThreads - 64;  // warps 2-9
-  constexpr int MAXST = BF ? 6 : 3;
+  constexpr int MAXST = BF ? 12 : 3;
   const int4 tl = tiles[blockIdx.x];
   const TcJob J = jobs[tl.x];
   const int mt = tl.w & 3;
@@ -429,7 +440,7 @@ __global__ void __launch_bounds__(kGramThreads, BF ? 2 : 1) k_gram_tc(const CUte
   const int nbox = kept_b > BM ? 2 : 1;      // 128-row TMA boxes of B
   // TF32: B head, B remainder (256 rows each) [, A head, A remainder];
   // BF16: 256 B rows [, 128 A rows], each split in place
-  constexpr int RING = BF ? RING_BYTES / 2 : RING_BYTES;  // BF16: two CTAs per SM
+  const int RING = BF ? ring : RING_BYTES;
   const int stage_bytes = BF ? (diag ? nbox * BM * RB : (BN + BM) * RB) : (diag ? 2 * B_BYTES : 2 * (B_BYTES + A_BYTES));
   const int stages = min(MAXST, RING / stage_bytes);  // TF32: 3 (diagonal) or 2; BF16: 6, 3 or 2
   const int a_off = BF ? BN * RB : 2 * B_BYTES;              // A rows of an off-diagonal stage
@@ -554,8 +565,8 @@ __global__ void __launch_bounds__(kGramThreads, BF ? 2 : 1) k_gram_tc(const CUte
         for (int k = 0; k < NSUB; ++k) {
           for (int q = 0; q < mt; ++q) {
             // diagonal: A sub-tile q is B rows [128 q, 128 q + 128)
-            const uint32_t ah = diag ? bh + q * A_BYTES : bh + 2 * B_BYTES;
-            const uint32_t al = diag ? bl + q * A_BYTES : bh + 2 * B_BYTES + A_BYTES;
+            const uint32_t ah = diag ? bh + (q0 + q) * A_BYTES : bh + 2 * B_BYTES;
+            const uint32_t al = diag ? bl + (q0 + q) * A_BYTES : bh + 2 * B_BYTES + A_BYTES;
             const uint32_t d = tmem + (uint32_t)(q * TMEM_COLS);
             mma<false>(d, sdesc(ah + k * 32), sdesc(bh + k * 32), id[q], (kb > 0 || k > 0) ? 1u : 0u);
             mma<false>(d, sdesc(ah + k * 32), sdesc(bl + k * 32), id[q], 1u);
@@ -571,11 +582,11 @@ __global__ void __launch_bounds__(kGramThreads, BF ? 2 : 1) k_gram_tc(const CUte
 
   // ---------------- epilogue: rows of D, and the transposes of the blocks
   // strictly below the diagonal (whose mirror images no tile computes);
-  // warps 0-3, one per 32 TMEM lanes
+  // warps 0-7, two per 32 TMEM lanes, each every other 32-column chunk
   const bool ok = mbar_wait(done, 0, abort, false);
   tc_fence_after();
-  if (warp >= 4) {
-    // no TMEM lanes of their own
+  if (warp >= 8) {
+    // no chunks of their own
   } else if (__all_sync(0xffffffffu, ok && !*abort)) {
     TO* stg = reinterpret_cast<TO*>(base) + warp * 32 * 33;
     TO* out = (CONTRACT ? reinterpret_cast<TO*>(out0)
@@ -584,14 +595,15 @@ __global__ void __launch_bounds__(kGramThreads, BF ? 2 : 1) k_gram_tc(const CUte
     const bool fpart = !CONTRACT && J.out_sel == 2;
     float* stgf = reinterpret_cast<float*>(base) + warp * 32 * 33;
     float* outf = fpart ? part + J.out_off : nullptr;
+    const int quad = warp & 3;
 #pragma unroll 1
     for (int sub = 0; sub < mt; ++sub) {
-      const int row0 = row_org + (q0 + sub) * BM + warp * 32;
+      const int row0 = row_org + (q0 + sub) * BM + quad * 32;
       const int cend = diag ? min(kept, BM * (q0 + sub + 1)) : kept;
 #pragma unroll 1
-      for (int c = 0; c * 32 < cend; ++c) {  // uniform over the warp
+      for (int c = warp >> 2; c * 32 < cend; c += 2) {  // uniform over the warp
         uint32_t v[32];
-        tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(sub * TMEM_COLS + c * 32), v);
+        tmem_ld32(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(sub * TMEM_COLS + c * 32), v);
         // strictly lower block of the symmetric Gram: its transpose is stored
         // too (the contraction's output is rectangular and has no mirror image)
         const bool mirror = !CONTRACT && (!diag || c < 4 * (q0 + sub));
@@ -601,10 +613,21 @@ __global__ void __launch_bounds__(kGramThreads, BF ? 2 : 1) k_gram_tc(const CUte
           __syncwarp();
           store_block(outf, stgf, J, lane, row0, col_org + c * 32, mirror);
         } else {
+          if constexpr (CONTRACT) {
 #pragma unroll
-          for (int q = 0; q < 32; ++q) {
-            if constexpr (CONTRACT) stg[lane * 33 + q] = __uint_as_float(v[q]);
-            else stg[lane * 33 + q] = widen_f32(v[q]);
+            for (int q = 0; q < 32; ++q) stg[lane * 33 + q] = __uint_as_float(v[q]);
+          } else {
+            bool sub_f32 = false;
+#pragma unroll
+            for (int q = 0; q < 32; ++q) {
+              stg[lane * 33 + q] = widen_normal_f32(v[q]);
+              sub_f32 = sub_f32 || subnormal_f32(v[q]);
+            }
+            if (sub_f32) {
+#pragma unroll
+              for (int q = 0; q < 32; ++q)
+                if (subnormal_f32(v[q])) stg[lane * 33 + q] = (double)__uint_as_float(v[q]);
+            }
           }
           __syncwarp();
           store_block(out, stg, J, lane, row0, col_org + c * 32, mirror);
@@ -716,6 +739,25 @@ gnmppi_status tc_plan_create(const std::vector<InstDesc>& desc, void* dRW, const
   std::vector<TcJob> chunk_jobs;  // appended after the 3 nb fixed jobs
   std::vector<GramRed> red;
   int64_t part_elems = 0;
+  int dev = 0, nsm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    err = "no device properties";
+    return GNMPPI_E_CUDA;
+  }
+  // Gram tiles with one sub-tile each: at most one per SM, or more
+  {
+    int64_t n1 = 0;
+    std::vector<int4> t;
+    for (auto& d : desc) {
+      t.clear();
+      gram_tiles(0, d.n, t, true);
+      n1 += (int64_t)t.size() * ((d.nR + kGramChunkCols - 1) / kGramChunkCols + (d.lsq ? 1 : 0));
+      if (n1 > nsm) break;
+    }
+    plan->few_g = n1 <= nsm;
+  }
+  const bool one_sub = bf16 != 0 || plan->few_g;
   for (int b = 0; b < nb; ++b) {
     const InstDesc& d = desc[b];
     if (d.ldK % KBLK != 0) {
@@ -791,7 +833,7 @@ gnmppi_status tc_plan_create(const std::vector<InstDesc>& desc, void* dRW, const
     const int gchunk = kGramChunkCols / KBLK;
     const int nchunks = (jg.nkb + gchunk - 1) / gchunk;
     if (nchunks <= 1) {
-      gram_tiles(nb + b, d.n, tg, bf16 != 0);
+      gram_tiles(nb + b, d.n, tg, one_sub);
     } else {
       const int64_t nn = (int64_t)d.n * d.n;
       for (int c = 0; c < nchunks; ++c) {
@@ -801,7 +843,7 @@ gnmppi_status tc_plan_create(const std::vector<InstDesc>& desc, void* dRW, const
         jc2.out_sel = 2;
         jc2.out_off = part_elems + c * nn;
         chunk_jobs.push_back(jc2);
-        gram_tiles(3 * nb + (int)chunk_jobs.size() - 1, d.n, tg, bf16 != 0);
+        gram_tiles(3 * nb + (int)chunk_jobs.size() - 1, d.n, tg, one_sub);
       }
       red.push_back(GramRed{d.o_nn, part_elems, nn, nchunks, b});
       part_elems += nchunks * nn;
@@ -812,7 +854,7 @@ gnmppi_status tc_plan_create(const std::vector<InstDesc>& desc, void* dRW, const
     js.map = 2 * nb + b;
     js.nkb = (d.n + KBLK - 1) / KBLK;
     js.out_sel = 1;
-    if (d.lsq) gram_tiles(2 * nb + b, d.n, ts, bf16 != 0);
+    if (d.lsq) gram_tiles(2 * nb + b, d.n, ts, one_sub);
   }
   // longest first, so that the short tiles (the S2 products, small
   // instances) fill the SMs that the last long ones leave idle.  Gram tiles
@@ -878,7 +920,7 @@ gnmppi_status tc_plan_create(const std::vector<InstDesc>& desc, void* dRW, const
   if (e == cudaSuccess && bf16)
     e = cudaFuncSetAttribute(k_contract_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, plan->smem1);
   if (e == cudaSuccess)
-    e = bf16 ? cudaFuncSetAttribute(k_gram_tc<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, plan->smem1)
+    e = bf16 ? cudaFuncSetAttribute(k_gram_tc<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, plan->smem)
              : cudaFuncSetAttribute(k_gram_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, plan->smem);
   if (e != cudaSuccess) {
     err = std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e);
@@ -903,19 +945,20 @@ cudaError_t tc_contract_launch(const TcPlan& plan, const InstState* d_st, float*
   else
     k_gram_tc<true><<<plan.ntiles_c, kGramThreads, plan.smem, stream>>>(plan.d_maps, plan.d_jobs, d_st,
                                                                         plan.d_tiles_c, P, nullptr, nullptr, plan.d_err,
-                                                                        inject);
+                                                                        inject, 0);
   return cudaGetLastError();
 }
 
 cudaError_t tc_gram_launch(const TcPlan& plan, const InstState* d_st, double* A, double* S2, cudaStream_t stream) {
   if (plan.ntiles_g == 0) return cudaSuccess;
+  const int ring = plan.few_g ? RING_BYTES : RING_BYTES / 2;
   if (plan.bf16)
-    k_gram_tc<false, true><<<plan.ntiles_g, kGramThreads, plan.smem1, stream>>>(
-        plan.d_maps, plan.d_jobs, d_st, plan.d_tiles_g, A, S2, plan.d_part, plan.d_err, 0);
+    k_gram_tc<false, true><<<plan.ntiles_g, kGramThreads, plan.few_g ? plan.smem : plan.smem1, stream>>>(
+        plan.d_maps, plan.d_jobs, d_st, plan.d_tiles_g, A, S2, plan.d_part, plan.d_err, 0, ring);
   else
     k_gram_tc<false><<<plan.ntiles_g, kGramThreads, plan.smem, stream>>>(plan.d_maps, plan.d_jobs, d_st,
                                                                           plan.d_tiles_g, A, S2, plan.d_part,
-                                                                          plan.d_err, 0);
+                                                                          plan.d_err, 0, ring);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && plan.nred > 0) {
     k_gram_reduce<<<dim3(32, plan.nred), 256, 0, stream>>>(plan.d_red, d_st, plan.d_part, A);

@@ -52,6 +52,7 @@ struct TcPlan {
   int ntiles_c = 0, ntiles_c1 = 0, ntiles_g = 0;
   int smem = 0, smem1 = 0;
   int max_nkb = 0;                // most k-blocks of a contraction tile
+  bool few_g = false;             // one-sub-tile Gram tiles fit one per SM
   int bf16 = 1;
   float* d_part = nullptr;        // FP32 chunk results of the chunked Grams
   GramRed* d_red = nullptr;       // one record per chunked instance
@@ -78,8 +79,8 @@ cudaError_t tc_contract_launch(const TcPlan& plan, const InstState* d_st, float*
 // mt without tuning: 1 where 256-row tiles would leave half the nsm SMs without
 // one, or where a tile is so short (K' <= 256) that starting up and storing it
 // weigh as much as its k-blocks; else 2.  mt = 2 against 1 (us): one chain of M =
-// 10 39 / 33, eight 41 / 35, 64 174 / 178; 256 at K' = 1024 657 / 657, at K' = 256
-// 278 / 252; 16 of M = 32 at K' = 2048 729 / 780.
+// 10 39 / 33, eight 39 / 35, 64 170 / 178; 256 at K' = 1024 636 / 658, at K' = 256
+// 260 / 252; 16 of M = 32 at K' = 2048 719 / 786.
 int tc_contract_default_mt(const TcPlan& plan, int nsm);
 
 // A = P^T P and, for instances in LSQ mode, S2 = S S^T (FP64 outputs) from
