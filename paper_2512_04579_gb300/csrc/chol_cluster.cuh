@@ -97,13 +97,6 @@ struct ClusterChol {
     return acc;
   }
 
-  // 1 / sqrt of a pivot; ok &= positive and finite, tested on the bits (a
-  // comparison would take a slot of the FP64 pipe in the serial chain).
-  static __device__ __forceinline__ double pivot(double d, bool& ok) {
-    const uint32_t hi = (uint32_t)__double2hiint(d);
-    ok = ok && hi < 0x7FF00000u && (hi | (uint32_t)__double2loint(d)) != 0u;
-    return rsqrt(d);
-  }
   // Step c of the diagonal factorisation on entry (r, k), k > c: col the scaled
   // column c, rj 1 / its pivot.
   static __device__ __forceinline__ double diag_step(double v, int r, int k, int c, double cr, double ck, double rj) {
@@ -130,7 +123,7 @@ struct ClusterChol {
       const int c0 = 2 * w, c1 = c0 + 1;
       double* col = m.col + (w & 1) * 34;
       if (warp == w) {
-        double rj = pivot(__shfl_sync(0xffffffffu, v, c0), ok);
+        double rj = pivot_rsqrt(__shfl_sync(0xffffffffu, v, c0), ok);
         if (k == c0) {
           v *= rj;
           col[r] = v;
@@ -139,7 +132,7 @@ struct ClusterChol {
         if (c1 < nb) {
           const double cr = __shfl_sync(0xffffffffu, v, r), ck = __shfl_sync(0xffffffffu, v, c1);
           if (k == c1) v = diag_step(v, r, k, c0, cr, ck, rj);
-          rj = pivot(__shfl_sync(0xffffffffu, v, 16 | c1), ok);
+          rj = pivot_rsqrt(__shfl_sync(0xffffffffu, v, 16 | c1), ok);
           if (k == c1) {
             v *= rj;
             col[17 + r] = v;

@@ -404,7 +404,8 @@ __device__ __forceinline__ double system_entry(const double* __restrict__ A, con
     const double sc = Keff * s[r] * s[r];
     t = (r == c) ? sc * sc : 0.0;
   }
-  return A[i] + lam * t + ((r == c && lsq) ? tau * A[i] : 0.0);
+  const double h = A[i] + lam * t;
+  return (r == c && lsq) ? __dadd_rn(h, __dmul_rn(tau, A[i])) : h;  // not contracted: retried systems keep their bits
 }
 __device__ __forceinline__ void build_system(const double* __restrict__ A, const double* __restrict__ S2,
                                              const double* __restrict__ s, bool lsq, double Keff, double lam,
@@ -511,7 +512,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_solve(SolveArgs a) {
     rhs[j] = -gj;
     gsq += gj * gj;
   }
-  gsq = block_sum(gsq, red);
+  gsq = block_sum_first(gsq, red);
   if (tid == 0) st.pr_norm = sqrt(gsq);  // |b|, b = P^T r
   double lam = a.cs.lambda;
   int retries = 0;
@@ -592,7 +593,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_solve(SolveArgs a) {
     }
     dsq += acc * acc;
   }
-  dsq = block_sum(dsq, red);
+  dsq = block_sum_first(dsq, red);
   if (tid == 0) {
     st.chol_retries = retries;
     st.lambda_used = lam;
