@@ -26,12 +26,12 @@ template <class Model, typename T, typename S>
 void launch_samples(const RollArgs& a, int nb, int smem, cudaStream_t s) {
   if (sizeof(T) == 8 && a.cs.sampling == 0) {
     const dim3 grid((unsigned)nb, (unsigned)((a.nmax * Model::NU + 1) / 2));
-    k_noise_f64<<<grid, a.cs.antithetic ? kPairsPerBlock : kSamplesPerBlock, 0, s>>>(a);
+    k_noise_f64<<<grid, sample_threads(true) / (a.cs.antithetic ? 2 : 1), 0, s>>>(a);
   }
   if (a.cs.antithetic)
-    k_samples<Model, T, S, true><<<nb, 128, smem, s>>>(a);
+    k_samples<Model, T, S, true><<<nb, sample_threads(sizeof(T) == 8), smem, s>>>(a);
   else
-    k_samples<Model, T, S, false><<<nb, 128, smem, s>>>(a);
+    k_samples<Model, T, S, false><<<nb, sample_threads(sizeof(T) == 8), smem, s>>>(a);
 }
 template <class Model, typename T, typename S>
 cudaError_t prepare_samples(int smem) {

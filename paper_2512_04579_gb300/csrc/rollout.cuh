@@ -133,7 +133,7 @@ struct SampleEmit {
 // here every pair of normals has a thread of its own (pendulum, N = 50, K = 256:
 // both kernels 259 us, 308 before; 64 instances 287, 310 before; chain M = 10
 // 4.72 ms, 4.83 before).
-static __global__ void __launch_bounds__(128) k_noise_f64(RollArgs a) {
+static __global__ void __launch_bounds__(64) k_noise_f64(RollArgs a) {
   const int2 bm = a.bmap[blockIdx.x];
   const InstDesc I = a.inst[bm.x];
   const int m = bm.y * (int)blockDim.x + threadIdx.x, j = 2 * blockIdx.y;
@@ -170,7 +170,7 @@ template <class Model, typename T, typename S, bool ANTI, bool FAST>
 __device__ __forceinline__ bool sample_rollout(const RollArgs& a, const InstDesc& I, int2 bm, const T* sU, const T* sS,
                                                const T* sR, const T* sRef) {
   constexpr int NX = Model::NX, NU = Model::NU;
-  const int per_block = ANTI ? kPairsPerBlock : kSamplesPerBlock;
+  constexpr int per_block = sample_threads(sizeof(T) == 8) / (ANTI ? 2 : 1);
   const int local = ANTI ? (threadIdx.x >> 1) : threadIdx.x;
   const int m = bm.y * per_block + local;
   const bool active = m < I.Kp;
@@ -302,7 +302,7 @@ __device__ __forceinline__ bool sample_rollout(const RollArgs& a, const InstDesc
 }
 
 template <class Model, typename T, typename S, bool ANTI>
-__global__ void __launch_bounds__(128) k_samples(RollArgs a) {
+__global__ void __launch_bounds__(sample_threads(sizeof(T) == 8)) k_samples(RollArgs a) {
   const int2 bm = a.bmap[blockIdx.x];
   const InstDesc I = a.inst[bm.x];
   if (a.st[bm.x].status != 0) return;
