@@ -261,7 +261,8 @@ const char* gnmppi_phase_name(int32_t i);
  * launch configurations and keeps the fastest:
  *   - branches: how many concurrent CUDA-graph branches carry the per-size
  *     rollout groups (sample rollouts and line search), 1, 2, 4 or 8;
- *   - solve_nt: threads per Cholesky CTA, 512 (one per SM), 256 (two) or 128
+ *   - solve_nt: threads per Cholesky CTA, 512 (one per SM; where the batch
+ *     leaves SMs idle, a cluster of such CTAs per instance), 256 (two) or 128
  *     (four); without tuning 512 when the batch fits one instance per SM, else 256.
  * reps: timed repetitions per candidate (<= 0: 3), after one warm-up.  The
  * choice is cached for the process under a signature of the device, the

@@ -41,7 +41,7 @@ constexpr int kMaxBranches = 8;
 // Launch configuration picked by the autotuner (or the defaults).
 struct TuneCfg {
   int branches = 1;   // concurrent graph branches for the per-size rollout groups
-  int solve_nt = 256; // threads per k_solve CTA (512: one CTA per SM, 256: two, 128: four)
+  int solve_nt = 256; // threads per k_solve CTA (512: one CTA per SM, or a cluster per instance where one fits, 256: two, 128: four)
   int contract_mt = 2; // BF16 contraction tile: A sub-tiles per CTA (2: one CTA per SM, 1: two)
 };
 
@@ -83,6 +83,9 @@ struct gnmppi_s {
   double* d_Hs = nullptr;
   int* d_cl_plan = nullptr;
   int64_t* d_o_cl = nullptr;
+  std::vector<int> cl_host;  // host copies until build's last synchronisation
+  std::vector<int64_t> cl_off_host;
+  std::vector<int2> grows_host, grows_lsq_host;
   bool use_tc = false;
   // concurrency of the rollout groups and the solve CTA shape
   TuneCfg tune{};
@@ -473,7 +476,7 @@ static gnmppi_status build(gnmppi_t h, const gnmppi_instance_shape* shapes) {
     CK(cudaMemcpyAsync(g.d_bmap, g.bmap.data(), sizeof(int2) * g.bmap.size(), cudaMemcpyHostToDevice, h->stream));
   }
   if (prec == kFP64) {
-    std::vector<int2> all_rows, lsq_rows;
+    std::vector<int2>&all_rows = h->grows_host, &lsq_rows = h->grows_lsq_host;
     for (int b = 0; b < h->batch; ++b) {
       const InstDesc& d = h->desc[b];
       h->nmax_u = std::max(h->nmax_u, d.n);
@@ -491,7 +494,6 @@ static gnmppi_status build(gnmppi_t h, const gnmppi_instance_shape* shapes) {
     if (!lsq_rows.empty())
       CK(cudaMemcpyAsync(h->d_grows_lsq, lsq_rows.data(), sizeof(int2) * lsq_rows.size(), cudaMemcpyHostToDevice,
                          h->stream));
-    CK(cudaStreamSynchronize(h->stream));  // the host vectors are temporaries
   }
 #undef AL
   // constants
@@ -567,6 +569,10 @@ static gnmppi_status build(gnmppi_t h, const gnmppi_instance_shape* shapes) {
   }
   set_branches(h, std::min<int>(4, (int)h->groups.size()));
   CK(cudaStreamSynchronize(h->stream));
+  h->cl_host = {};
+  h->cl_off_host = {};
+  h->grows_host = {};
+  h->grows_lsq_host = {};
   return GNMPPI_OK;
 }
 
@@ -697,20 +703,21 @@ static cudaLaunchConfig_t cluster_config(int cs, int batch, int smem, cudaStream
   return cfg;
 }
 
-// Clusters of cs CTAs that the device holds at once (0: none, or the attributes are refused).
+// Whether the device holds `batch` clusters of cs CTAs at once; opts the kernel
+// in.  Portable sizes that take at most half the SMs need no query.
 template <typename TA>
-static int cluster_capacity(int cs, int smem) {
+static bool cluster_fits(int cs, int batch, int smem, int nsm) {
   auto k = k_solve_cluster<TA>;
-  int n = 0;
+  int n = batch;
   cudaLaunchAttribute attr;
   const cudaLaunchConfig_t cfg = cluster_config(cs, 1, smem, nullptr, &attr);
   if (raise_smem(k, smem) != cudaSuccess ||
       (cs > 8 && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
-      cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
+      ((cs > 8 || 2 * cs * batch > nsm) && cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess)) {
     cudaGetLastError();
-    return 0;
+    return false;
   }
-  return n;
+  return n >= batch;
 }
 
 template <typename TA>
@@ -750,15 +757,16 @@ static gnmppi_status choose_cluster(gnmppi_t h, int optin, int nsm) {
   size_t k = 0;
   while (k + 1 < sizes.size() && sizes[k + 1].path <= 1.02 * best) ++k;
   for (; k < sizes.size() && !h->cl_size; ++k) {
-    const int cap = h->p.precision == kFP64 ? cluster_capacity<double>(sizes[k].cs, sizes[k].smem)
-                                            : cluster_capacity<float>(sizes[k].cs, sizes[k].smem);
-    if (cap < h->batch) continue;
+    if (!(h->p.precision == kFP64 ? cluster_fits<double>(sizes[k].cs, h->batch, sizes[k].smem, nsm)
+                                  : cluster_fits<float>(sizes[k].cs, h->batch, sizes[k].smem, nsm)))
+      continue;
     h->cl_size = sizes[k].cs;
     h->cl_smem = sizes[k].smem;
   }
   if (!h->cl_size) return GNMPPI_OK;
-  std::vector<int> all;
-  std::vector<int64_t> off(h->batch);
+  std::vector<int>& all = h->cl_host;
+  std::vector<int64_t>& off = h->cl_off_host;
+  off.resize(h->batch);
   std::map<int, std::vector<int>> by_n;
   for (int b = 0; b < h->batch; ++b) {
     const int n = h->desc[b].n;
@@ -776,7 +784,6 @@ static gnmppi_status choose_cluster(gnmppi_t h, int optin, int nsm) {
   if ((st = dalloc(h, &h->d_o_cl, sizeof(int64_t) * off.size())) != GNMPPI_OK) return st;
   CK(cudaMemcpyAsync(h->d_cl_plan, all.data(), sizeof(int) * all.size(), cudaMemcpyHostToDevice, h->stream));
   CK(cudaMemcpyAsync(h->d_o_cl, off.data(), sizeof(int64_t) * off.size(), cudaMemcpyHostToDevice, h->stream));
-  CK(cudaStreamSynchronize(h->stream));  // the host vectors are temporaries
   return GNMPPI_OK;
 }
 
