@@ -113,17 +113,6 @@ struct gnmppi_s {
   std::string err;
 };
 
-// Opt kernel k into at least `smem` bytes of dynamic shared memory.  The
-// attribute belongs to the function, not to a handle, so it is only ever
-// raised: another handle may have opted in to more.
-template <typename K>
-static cudaError_t raise_smem(K k, int smem) {
-  cudaFuncAttributes at{};
-  cudaError_t e = cudaFuncGetAttributes(&at, k);
-  if (e != cudaSuccess || at.maxDynamicSharedSizeBytes >= smem) return e;
-  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-}
-
 static thread_local std::string g_create_err;  // errors raised before a handle exists
 
 static void assign_branches(gnmppi_t h, int nb);
@@ -535,18 +524,18 @@ static gnmppi_status build(gnmppi_t h, const gnmppi_instance_shape* shapes) {
     const int pct4 = std::min(100, (int)(100.0 * 4 * (h->solve_smem + 2048) / std::max(1, smsm)) + 5);
     const int pct1 = std::min(100, (int)(100.0 * (h->solve_smem + 2048) / std::max(1, smsm)) + 5);
     if (prec == kFP64) {
-      CK(cudaFuncSetAttribute(k_solve<double, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, h->solve_smem));
+      CK(raise_smem(k_solve<double, 512>, h->solve_smem));
       CK(cudaFuncSetAttribute(k_solve<double, 512>, cudaFuncAttributePreferredSharedMemoryCarveout, pct1));
-      CK(cudaFuncSetAttribute(k_solve<double, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, h->solve_smem));
+      CK(raise_smem(k_solve<double, 256>, h->solve_smem));
       CK(cudaFuncSetAttribute(k_solve<double, 256>, cudaFuncAttributePreferredSharedMemoryCarveout, pct2));
-      CK(cudaFuncSetAttribute(k_solve<double, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, h->solve_smem));
+      CK(raise_smem(k_solve<double, 128>, h->solve_smem));
       CK(cudaFuncSetAttribute(k_solve<double, 128>, cudaFuncAttributePreferredSharedMemoryCarveout, pct4));
     } else {
-      CK(cudaFuncSetAttribute(k_solve<float, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, h->solve_smem));
+      CK(raise_smem(k_solve<float, 512>, h->solve_smem));
       CK(cudaFuncSetAttribute(k_solve<float, 512>, cudaFuncAttributePreferredSharedMemoryCarveout, pct1));
-      CK(cudaFuncSetAttribute(k_solve<float, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, h->solve_smem));
+      CK(raise_smem(k_solve<float, 256>, h->solve_smem));
       CK(cudaFuncSetAttribute(k_solve<float, 256>, cudaFuncAttributePreferredSharedMemoryCarveout, pct2));
-      CK(cudaFuncSetAttribute(k_solve<float, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, h->solve_smem));
+      CK(raise_smem(k_solve<float, 128>, h->solve_smem));
       CK(cudaFuncSetAttribute(k_solve<float, 128>, cudaFuncAttributePreferredSharedMemoryCarveout, pct4));
     }
   }

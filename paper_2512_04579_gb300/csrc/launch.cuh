@@ -22,6 +22,17 @@ bool launchers_f32(int dyn, int key, Launchers* out);
 bool group_launchers_f64(int F, Launchers* out);
 bool group_launchers_f32(int F, Launchers* out);
 
+// Opt kernel k into at least `smem` bytes of dynamic shared memory.  The
+// attribute belongs to the function, not to a handle, so it is only ever
+// raised: another handle may have opted in to more.
+template <typename K>
+cudaError_t raise_smem(K k, int smem) {
+  cudaFuncAttributes at{};
+  cudaError_t e = cudaFuncGetAttributes(&at, k);
+  if (e != cudaSuccess || at.maxDynamicSharedSizeBytes >= smem) return e;
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+}
+
 template <class Model, typename T, typename S>
 void launch_samples(const RollArgs& a, int nb, int smem, cudaStream_t s) {
   if (sizeof(T) == 8 && a.cs.sampling == 0) {
@@ -35,9 +46,8 @@ void launch_samples(const RollArgs& a, int nb, int smem, cudaStream_t s) {
 }
 template <class Model, typename T, typename S>
 cudaError_t prepare_samples(int smem) {
-  cudaError_t e = cudaFuncSetAttribute(k_samples<Model, T, S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_samples<Model, T, S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const cudaError_t e = raise_smem(k_samples<Model, T, S, true>, smem);
+  return e != cudaSuccess ? e : raise_smem(k_samples<Model, T, S, false>, smem);
 }
 template <class Model, typename T>
 void launch_line(const RollArgs& a, int nthreads, cudaStream_t s) {

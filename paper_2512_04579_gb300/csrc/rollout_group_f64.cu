@@ -6,7 +6,7 @@ namespace gnm {
 namespace {
 template <typename T, typename S, int FL, int G>
 cudaError_t prep(int smem) {
-  return cudaFuncSetAttribute(k_samples_group<T, S, FL, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  return raise_smem(k_samples_group<T, S, FL, G>, smem);
 }
 template <typename T, typename S, int FL, int G>
 void samp(const RollArgs& a, int nb, int smem, cudaStream_t s) {
