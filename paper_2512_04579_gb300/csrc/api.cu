@@ -83,8 +83,7 @@ struct gnmppi_s {
   double* d_Hs = nullptr;
   int* d_cl_plan = nullptr;
   int64_t* d_o_cl = nullptr;
-  std::vector<int> cl_host;  // host copies until build's last synchronisation
-  std::vector<int64_t> cl_off_host;
+  std::vector<int64_t> cl_host;  // host copies until build's last synchronisation
   std::vector<int2> grows_host, grows_lsq_host;
   bool use_tc = false;
   // concurrency of the rollout groups and the solve CTA shape
@@ -559,7 +558,6 @@ static gnmppi_status build(gnmppi_t h, const gnmppi_instance_shape* shapes) {
   set_branches(h, std::min<int>(4, (int)h->groups.size()));
   CK(cudaStreamSynchronize(h->stream));
   h->cl_host = {};
-  h->cl_off_host = {};
   h->grows_host = {};
   h->grows_lsq_host = {};
   return GNMPPI_OK;
@@ -753,8 +751,8 @@ static gnmppi_status choose_cluster(gnmppi_t h, int optin, int nsm) {
     h->cl_smem = sizes[k].smem;
   }
   if (!h->cl_size) return GNMPPI_OK;
-  std::vector<int>& all = h->cl_host;
-  std::vector<int64_t>& off = h->cl_off_host;
+  std::vector<int> all;
+  std::vector<int64_t>& off = h->cl_host;
   off.resize(h->batch);
   std::map<int, std::vector<int>> by_n;
   for (int b = 0; b < h->batch; ++b) {
@@ -768,11 +766,14 @@ static gnmppi_status choose_cluster(gnmppi_t h, int optin, int nsm) {
     all.insert(all.end(), q.begin(), q.end());
   }
   gnmppi_status st;
-  if ((st = dalloc(h, &h->d_Hs, 8 * h->n_nn)) != GNMPPI_OK) return st;
-  if ((st = dalloc(h, &h->d_cl_plan, sizeof(int) * all.size())) != GNMPPI_OK) return st;
-  if ((st = dalloc(h, &h->d_o_cl, sizeof(int64_t) * off.size())) != GNMPPI_OK) return st;
-  CK(cudaMemcpyAsync(h->d_cl_plan, all.data(), sizeof(int) * all.size(), cudaMemcpyHostToDevice, h->stream));
-  CK(cudaMemcpyAsync(h->d_o_cl, off.data(), sizeof(int64_t) * off.size(), cudaMemcpyHostToDevice, h->stream));
+  // one allocation: the systems, the plans' offsets, the plans
+  const size_t words = off.size() + (all.size() + 1) / 2;
+  if ((st = dalloc(h, &h->d_Hs, 8 * (h->n_nn + words))) != GNMPPI_OK) return st;
+  h->d_o_cl = reinterpret_cast<int64_t*>(h->d_Hs + h->n_nn);
+  h->d_cl_plan = reinterpret_cast<int*>(h->d_o_cl + off.size());
+  off.resize(words);
+  memcpy(off.data() + h->batch, all.data(), sizeof(int) * all.size());
+  CK(cudaMemcpyAsync(h->d_o_cl, off.data(), 8 * words, cudaMemcpyHostToDevice, h->stream));
   return GNMPPI_OK;
 }
 
