@@ -17,17 +17,12 @@
 // bitwise those of the single-CTA kernel.
 #pragma once
 #include "chol.cuh"
+#include "cluster_plan.cuh"
 
 namespace gnm {
 
 constexpr int kClThreads = 512;
-constexpr int kClMaxBlocks = 256;  // block rows of 16 an instance may have (n <= 4096; shared memory sets less)
-
-// Row plan entry of block row I (host-made, cluster_plan): owning rank and the
-// index of the row's first block in the rank's block storage.
-__host__ __device__ __forceinline__ int cl_entry(int rank, int slot) { return (rank << 24) | slot; }
-__device__ __forceinline__ int cl_rank(int e) { return e >> 24; }
-__device__ __forceinline__ int cl_slot(int e) { return e & 0xFFFFFF; }
+static_assert(CNB == kClBlock, "the row plans count blocks of the panel width");
 
 __device__ __forceinline__ void cl_arrive() {
   __syncwarp();
@@ -62,9 +57,6 @@ struct ClSmem {
   double* pbuf;  // [nblk][256] the panel's L blocks; after the factorisation the vectors (ClVec)
   double* blk;   // this rank's block rows: A, then L, with the inverse of the diagonal block in its place
 };
-__host__ __device__ inline int64_t cl_fixed_doubles(int n) {
-  return 512 + 1024 + 256 + 68 + (int64_t)((n + 15) / 16) * 256;
-}
 
 // Vectors of n doubles that take the panel buffer's place (16 n doubles).
 struct ClVec {
@@ -79,7 +71,7 @@ struct ClusterChol {
   ClSmem m;
   const int* plan;   // [nblk]
   const int* rows;   // shared memory: this rank's block rows, ascending
-  int* fail;         // shared memory, one per rank
+  int* fail;         // shared memory [2]: failed diagonal blocks (cl_fail_word)
   int n, nblk, nrows, rank, size;
   bool rank0_rows;   // rank 0 owns block rows (and so needs the panels)
 
@@ -150,7 +142,7 @@ struct ClusterChol {
 #pragma unroll 4
     for (int q = 0; q < size; ++q) cl_map(m.ybuf, q)[(d & 1) * 256 + k * CNB + r] = y;
     if (!ok && (t & 31) == 0)
-      for (int q = 0; q < size; ++q) *cl_map(fail, q) = 1;
+      for (int q = 0; q < size; ++q) *cl_map(fail + cl_fail_word(d), q) = 1;
   }
 
   // Rank 0, threads t < 256: from the buffered blocks of panel p, L of block
@@ -247,8 +239,8 @@ struct ClusterChol {
   template <class Entry>
   __device__ bool factor(double* H, const Entry& entry) {
     const int t = threadIdx.x;
-    __syncthreads();  // every thread has read the last attempt's flag
-    if (t == 0) *fail = 0;
+    __syncthreads();  // every thread has read the last attempt's flags
+    if (t == 0) fail[0] = fail[1] = 0;
     for (int x = 0; x < nrows; ++x) {
       const int I = rows[x];
       double* row = block(I, 0);
@@ -286,7 +278,7 @@ struct ClusterChol {
     if (rank == 0 && t < 256) diag(0, v);
     cl_arrive();
     cl_wait();
-    if (*fail) return false;
+    if (fail[cl_fail_word(0)]) return false;
     for (int p = 0; p + 1 < nblk; ++p) {
       panel(p);
       cl_arrive();
@@ -295,7 +287,7 @@ struct ClusterChol {
       trailing(p);
       cl_arrive();
       cl_wait();
-      if (*fail) return false;
+      if (fail[cl_fail_word(p + 1)]) return false;
     }
     keep_inverse(nblk - 1);
     return true;
@@ -447,47 +439,5 @@ struct ClusterChol {
              (((double)l[0] + (double)l[1]) + ((double)l[2] + (double)l[3]));
   }
 };
-
-// Host side: row plans of an n x n system over cs ranks.  A block update (16^3
-// DFMA) takes about 2600 cycles of an SM's FP64 pipe, rank 0's chain per panel
-// 18600 (its 16 pivot columns run one after another, about 900 cycles each),
-// seven block updates; so rank 0 starts with that load and the rows go, longest
-// first, to the least loaded rank.
-constexpr int kClChainBlocks = 7;
-inline int cluster_plan(int n, int cs, int* plan) {  // returns the most blocks a rank stores
-  const int nblk = (n + CNB - 1) / CNB;
-  long load[16] = {0};
-  int slots[16] = {0};
-  load[0] = (long)kClChainBlocks * nblk;
-  for (int I = nblk - 1; I >= 0; --I) {
-    int q = 0;
-    for (int k = 1; k < cs; ++k)
-      if (load[k] < load[q]) q = k;
-    plan[I] = cl_entry(q, slots[q]);
-    slots[q] += I + 1;
-    load[q] += (long)I * (I + 1) / 2 + 1;
-  }
-  int most = 0, rows[16] = {0};
-  for (int I = 0; I < nblk; ++I)
-    if (++rows[plan[I] >> 24] > 32) return 1 << 20;  // half warps of a CTA
-  for (int k = 0; k < cs; ++k) most = slots[k] > most ? slots[k] : most;
-  return most;
-}
-// Block updates of the longest path through the factorisation (plan of n, cs).
-inline long cluster_path(int n, int cs, const int* plan) {
-  const int nblk = (n + CNB - 1) / CNB;
-  long path = 0;
-  for (int p = 0; p + 1 < nblk; ++p) {
-    long load[16] = {kClChainBlocks};
-    long worst = kClChainBlocks;
-    for (int I = p + 2; I < nblk; ++I) {
-      long& l = load[plan[I] >> 24];
-      l += I - p;
-      worst = l > worst ? l : worst;
-    }
-    path += worst + 2;  // + the panel's own blocks and the two barriers
-  }
-  return path;
-}
 
 }  // namespace gnm

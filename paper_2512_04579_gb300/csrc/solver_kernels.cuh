@@ -614,7 +614,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_solve_cluster(SolveArgs a) {
   const InstDesc I = a.inst[b];
   const int n = I.n, tid = threadIdx.x;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int fail, nrows;
+  __shared__ int fail[2], nrows;
   __shared__ int rows[kClMaxBlocks];
   __shared__ double red[32];
   ClusterChol cc;
@@ -624,7 +624,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_solve_cluster(SolveArgs a) {
   cc.rank = cl_my_rank();
   cc.plan = a.cl_plan + a.o_cl[b];
   cc.rows = rows;
-  cc.fail = &fail;
+  cc.fail = fail;
   double* v = reinterpret_cast<double*>(smem_raw);
   cc.m.ybuf = v;
   cc.m.cbuf = v + 512;
