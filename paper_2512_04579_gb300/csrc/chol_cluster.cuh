@@ -24,11 +24,21 @@ namespace gnm {
 constexpr int kClThreads = 512;
 static_assert(CNB == kClBlock, "the row plans count blocks of the panel width");
 
+// The barriers below are .aligned: a warp's threads execute them together, so
+// each first brings the warp's threads back together.
 __device__ __forceinline__ void cl_arrive() {
   __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void cl_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cl_wait() {
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Barrier `id` of eight warps of the CTA.
+__device__ __forceinline__ void bar_256(int id) {
+  __syncwarp();
+  asm volatile("bar.sync %0, 256;" ::"r"(id) : "memory");
+}
 __device__ __forceinline__ int cl_size() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
@@ -132,7 +142,7 @@ struct ClusterChol {
           }
         }
       }
-      asm volatile("bar.sync 1, 256;" ::: "memory");
+      bar_256(1);
       if (k > c1) {
         v = diag_step(v, r, k, c0, col[r], col[k], col[16]);
         if (c1 < nb) v = diag_step(v, r, k, c1, col[17 + r], col[17 + k], col[33]);
@@ -153,7 +163,7 @@ struct ClusterChol {
     int r, c;
     const double l = panel_entry(A1, m.ybuf + (p & 1) * 256, t, r, c);
     m.lbuf[c * 16 + r] = l;
-    asm volatile("bar.sync 1, 256;" ::: "memory");
+    bar_256(1);
     r = t & 15;
     const int k = t >> 4;
     double v = 0.0;
@@ -184,7 +194,7 @@ struct ClusterChol {
       const double l = panel_entry(at, m.ybuf + (p & 1) * 256, t, r, c);
 #pragma unroll 4
       for (int q = rank0_rows ? 0 : 1; q < size; ++q) cl_map(m.pbuf, q)[I * 256 + c * 16 + r] = l;
-      asm volatile("bar.sync %0, 256;" ::"r"(2 + half) : "memory");  // the half's threads have read the block
+      bar_256(2 + half);  // the half's threads have read the block
       at[c * 16 + r] = l;
     }
   }

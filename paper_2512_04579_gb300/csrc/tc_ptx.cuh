@@ -117,8 +117,10 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
                    "=r"(x[22]), "=r"(x[23]), "=r"(x[24]), "=r"(x[25]), "=r"(x[26]), "=r"(x[27]), "=r"(x[28]),     \
                    "=r"(x[29]), "=r"(x[30]), "=r"(x[31])
 
-// 32 consecutive TMEM columns of this thread's lane.
+// 32 consecutive TMEM columns of this thread's lane.  The load is .aligned, and
+// its callers' loops branch per lane (stores of live rows only).
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* v) {
+  __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
       "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
