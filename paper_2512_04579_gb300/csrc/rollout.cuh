@@ -289,6 +289,7 @@ __device__ __forceinline__ bool sample_rollout(const RollArgs& a, const InstDesc
     ev += __shfl_xor_sync(0xffffffffu, ev, 1);
   }
   const bool ok = isfinite(Cself) && isfinite(Cother) && isfinite(ev);
+  __syncwarp();  // the partner lane's stores come before the zeros that replace them
   if (active && GNM_IN(m, I.Kp)) {
     a.C[I.o_C + (ANTI ? 2 * m + par : m)] = Cself;
     if (par == 0) a.e[I.o_C / 2 + m] = ok ? ev : 0.0;
@@ -322,8 +323,10 @@ __global__ void __launch_bounds__(sample_threads(sizeof(T) == 8)) k_samples(Roll
   __syncthreads();
   const bool ok = sample_rollout<Model, T, S, ANTI, true>(a, I, bm, sU, sS, sR, sRef);
   if constexpr (HasFast<Model>::value) {
-    if (__any_sync(0xffffffffu, !ok))  // a subnormal link length, or a diverged rollout
+    if (__any_sync(0xffffffffu, !ok)) {  // a subnormal link length, or a diverged rollout
+      __syncwarp();  // the first pass's zeros of other lanes come before the values that replace them
       sample_rollout<Model, T, S, ANTI, false>(a, I, bm, sU, sS, sR, sRef);
+    }
   }
 }
 

@@ -419,6 +419,7 @@ __device__ __forceinline__ bool group_rollout(const RollArgs& a, const InstDesc&
     a.C[I.o_C + 2 * m + (plus ? 0 : 1)] = Cself;
     if (plus) a.e[I.o_C / 2 + m] = ok ? ev : 0.0;
   }
+  __syncwarp();  // the other lanes' stores come before the zeros that replace them
   if (active && plus && !ok) {  // dropped pair: its columns leave P and S
     const int rows = I.N * rps + 2 * I.F;
     for (int row = lg; row < rows; row += G) put(dR + (int64_t)row * I.ldK + m, (T)0);
@@ -469,8 +470,10 @@ __global__ void __launch_bounds__(256, 2) k_samples_group(RollArgs a) {
   __syncthreads();
 
   const bool ok = group_rollout<T, S, FL, G, FX, true>(a, I, bm, sU, sS, sR, sRef);
-  if (sizeof(T) == 4 && __any_sync(0xffffffffu, !ok))  // a subnormal link length, or a diverged rollout
+  if (sizeof(T) == 4 && __any_sync(0xffffffffu, !ok)) {  // a subnormal link length, or a diverged rollout
+    __syncwarp();  // the first pass's zeros of other lanes come before the values that replace them
     group_rollout<T, S, FL, G, FX, false>(a, I, bm, sU, sS, sR, sRef);
+  }
 }
 
 // Line search / nominal / FP64 cost for groups: one group per (instance, candidate).
