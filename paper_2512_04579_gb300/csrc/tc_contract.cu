@@ -60,6 +60,10 @@ constexpr int KBLK = 32;        // k-block: 32 FP32 values, or their 32 BF16 hea
 constexpr int A_BYTES = BM * ROW_BYTES;
 constexpr int B_BYTES = BN * ROW_BYTES;
 constexpr int RING_BYTES = 4 * (A_BYTES + B_BYTES);  // 192 KB of operand ring (every kernel here)
+// Shared memory beside the ring: up to 1023 bytes to align it, and the words
+// behind it (three barriers per stage, the final one, TMEM slot, abort word).
+constexpr int ALIGN_BYTES = 1024, WORD_BYTES = 512;
+constexpr bool words_fit(int stages) { return (3 * stages + 1) * 8 + 2 * 4 <= WORD_BYTES; }
 constexpr int TMEM_COLS = 256;
 
 // BF16 heads of two adjacent FP32 values (round to nearest even) and the
@@ -145,6 +149,7 @@ __global__ void __launch_bounds__(kContractThreads<MT>, 3 - MT) k_contract_tc(co
   constexpr int TILE = A_BYTES;              // one landed 128-row box (16 KB)
   constexpr int STAGE_BYTES = (MT + 2) * TILE;  // A sub-tiles, then 256 B rows
   constexpr int STAGES = (MT == 2 ? RING_BYTES : RING_BYTES / 2) / STAGE_BYTES;
+  static_assert(words_fit(STAGES), "barriers, TMEM slot and abort word overrun their reserve");
   constexpr int SPLITTERS = MT * BM;
   constexpr uint32_t TCOLS = MT * TMEM_COLS;
   const int4 tl = tiles[blockIdx.x];
@@ -429,6 +434,7 @@ __global__ void __launch_bounds__(kGramThreads, BF ? 2 : 1) k_gram_tc(const CUte
   constexpr int RB = ROW_BYTES;  // bytes of one landed row of a k-block
   constexpr int SPLITTERS = kGramThreads - 64;  // warps 2-9
   constexpr int MAXST = BF ? 12 : 3;
+  static_assert(words_fit(MAXST), "barriers, TMEM slot and abort word overrun their reserve");
   const int4 tl = tiles[blockIdx.x];
   const TcJob J = jobs[tl.x];
   const int mt = tl.w & 3;
@@ -913,8 +919,8 @@ gnmppi_status tc_plan_create(const std::vector<InstDesc>& desc, void* dRW, const
     err = "copying the tensor-core plan failed";
     return GNMPPI_E_CUDA;
   }
-  plan->smem = RING_BYTES + 1024 + 256;
-  plan->smem1 = RING_BYTES / 2 + 1024 + 256;
+  plan->smem = RING_BYTES + ALIGN_BYTES + WORD_BYTES;
+  plan->smem1 = RING_BYTES / 2 + ALIGN_BYTES + WORD_BYTES;
   cudaError_t e = bf16 ? cudaFuncSetAttribute(k_contract_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, plan->smem)
                        : cudaFuncSetAttribute(k_gram_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, plan->smem);
   if (e == cudaSuccess && bf16)
