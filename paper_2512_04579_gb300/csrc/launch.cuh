@@ -2,6 +2,7 @@
 // Internal; one table per rollout precision (rollout_{f64,f32}.cu).
 #pragma once
 #include "rollout_group.cuh"
+#include "smem_limit.cuh"
 
 namespace gnm {
 
@@ -22,15 +23,17 @@ bool launchers_f32(int dyn, int key, Launchers* out);
 bool group_launchers_f64(int F, Launchers* out);
 bool group_launchers_f32(int F, Launchers* out);
 
-// Opt kernel k into at least `smem` bytes of dynamic shared memory.  The
-// attribute belongs to the function, not to a handle, so it is only ever
-// raised: another handle may have opted in to more.
+// Opt kernel k into at least `smem` bytes of dynamic shared memory.
 template <typename K>
 cudaError_t raise_smem(K k, int smem) {
-  cudaFuncAttributes at{};
-  cudaError_t e = cudaFuncGetAttributes(&at, k);
-  if (e != cudaSuccess || at.maxDynamicSharedSizeBytes >= smem) return e;
-  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  return raise_limit(
+      [&](int* current) {
+        cudaFuncAttributes at{};
+        const cudaError_t e = cudaFuncGetAttributes(&at, k);
+        *current = at.maxDynamicSharedSizeBytes;
+        return e;
+      },
+      [&](int bytes) { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); }, smem);
 }
 
 template <class Model, typename T, typename S>
