@@ -283,7 +283,8 @@ gnmppi_status gnmppi_autotune(gnmppi_t h, int32_t mem, const double* x0, const d
 gnmppi_status gnmppi_tune_set(gnmppi_t h, int32_t branches, int32_t solve_nt, int32_t contract_mt);
 
 /* The handle's launch configuration as a JSON object (source "default",
- * "set", "cache" or "timed"; the timed candidates when tuned), NUL-terminated
+ * "set", "cache" or "timed"; the timed candidates when tuned; solve_ctas: the
+ * CTAs that share one instance's damped solve, 1 without a cluster), NUL-terminated
  * into buf (host, cap bytes).  Errors: E_ARG if cap is too small. */
 gnmppi_status gnmppi_tune_report(gnmppi_t h, char* buf, int32_t cap);
 

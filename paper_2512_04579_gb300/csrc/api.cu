@@ -1490,6 +1490,8 @@ extern "C" gnmppi_status gnmppi_debug_inject(gnmppi_t h, int32_t kind, int32_t i
   return GNMPPI_OK;
 }
 
+static int solve_ctas(gnmppi_t h) { return h->tune.solve_nt == 512 && h->cl_size ? h->cl_size : 1; }
+
 extern "C" gnmppi_status gnmppi_tune_report(gnmppi_t h, char* buf, int32_t cap) {
   if (!h || !buf || cap <= 0) return GNMPPI_E_ARG;
   std::string r = h->tune_report;
@@ -1499,6 +1501,8 @@ extern "C" gnmppi_status gnmppi_tune_report(gnmppi_t h, char* buf, int32_t cap) 
              h->tune.branches, h->tune.solve_nt, h->tune.contract_mt);
     r = b;
   }
+  // CTAs per instance of the solve as it is configured now
+  r.insert(r.size() - 1, ", \"solve_ctas\": " + std::to_string(solve_ctas(h)));
   if ((int32_t)r.size() + 1 > cap) return fail(h, GNMPPI_E_ARG, "report needs %d bytes", (int)r.size() + 1);
   memcpy(buf, r.c_str(), r.size() + 1);
   return GNMPPI_OK;
