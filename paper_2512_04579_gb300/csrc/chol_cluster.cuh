@@ -49,7 +49,16 @@ __device__ __forceinline__ int cl_my_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return (int)r;
 }
+// Doubles of dynamic shared memory this CTA was launched with.
+__device__ __forceinline__ int64_t cl_dyn_words() {
+  uint32_t r;
+  asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(r));
+  return (int64_t)(r / 8);
+}
 // The shared-memory object that p is in this CTA, in the CTA of the given rank.
+// A remote address is always this function's result or an index from it: one
+// formed by adding a distance to a pointer into this CTA's shared memory would be
+// stored to as this CTA's.
 template <typename T>
 __device__ __forceinline__ T* cl_map(T* p, int rank) {
   uint64_t q;
@@ -58,14 +67,22 @@ __device__ __forceinline__ T* cl_map(T* p, int rank) {
 }
 
 // Shared memory of a cluster CTA, in doubles from a 16-byte aligned base.
-// Blocks are stored column by column (entry (r, c) at 16 c + r).
+// Blocks are stored column by column (entry (r, c) at 16 c + r).  Stores test
+// their address against `words`, the CTA's dynamic shared memory, in the
+// bounds-check build (has(); the CTAs of a cluster all have as much, so a store
+// to another rank tests the address it was mapped from).
 struct ClSmem {
+  int64_t words;
   double* ybuf;  // [2][256] inverted diagonal blocks (row-major), by panel parity
   double* cbuf;  // [2][512] rank 0: blocks (p+1, p) and (p+1, p+1) of panel p, by parity
   double* lbuf;  // [256] rank 0: L of block (p+1, p)
   double* col;   // [2][34] rank 0: two columns of the diagonal factor, each with 1 / its pivot
   double* pbuf;  // [nblk][256] the panel's L blocks; after the factorisation the vectors (ClVec)
   double* blk;   // this rank's block rows: A, then L, with the inverse of the diagonal block in its place
+  template <typename V>
+  __device__ __forceinline__ bool has(const V* p) const {
+    return GNM_IN(reinterpret_cast<const char*>(p) - reinterpret_cast<const char*>(ybuf), 8 * words - (int64_t)sizeof(V) + 1);
+  }
 };
 
 // Vectors of n doubles that take the panel buffer's place (16 n doubles).
@@ -128,7 +145,7 @@ struct ClusterChol {
         double rj = pivot_rsqrt(__shfl_sync(0xffffffffu, v, c0), ok);
         if (k == c0) {
           v *= rj;
-          col[r] = v;
+          if (m.has(col + r)) col[r] = v;
           if (r == c0) col[16] = rinv = rj;
         }
         if (c1 < nb) {
@@ -137,7 +154,7 @@ struct ClusterChol {
           rj = pivot_rsqrt(__shfl_sync(0xffffffffu, v, 16 | c1), ok);
           if (k == c1) {
             v *= rj;
-            col[17 + r] = v;
+            if (m.has(col + 17 + r)) col[17 + r] = v;
             if (r == c1) col[33] = rinv = rj;
           }
         }
@@ -149,8 +166,11 @@ struct ClusterChol {
       }
     }
     const double y = r < k ? v : (r == k ? rinv : 0.0);  // inverse entry (k, r)
+    double* yd = m.ybuf + (d & 1) * 256 + k * CNB + r;
+    if (m.has(yd)) {
 #pragma unroll 4
-    for (int q = 0; q < size; ++q) cl_map(m.ybuf, q)[(d & 1) * 256 + k * CNB + r] = y;
+      for (int q = 0; q < size; ++q) *cl_map(yd, q) = y;
+    }
     if (!ok && (t & 31) == 0)
       for (int q = 0; q < size; ++q) *cl_map(fail + cl_fail_word(d), q) = 1;
   }
@@ -162,7 +182,7 @@ struct ClusterChol {
     const double* A1 = m.cbuf + (p & 1) * 512;
     int r, c;
     const double l = panel_entry(A1, m.ybuf + (p & 1) * 256, t, r, c);
-    m.lbuf[c * 16 + r] = l;
+    if (m.has(m.lbuf + c * 16 + r)) m.lbuf[c * 16 + r] = l;
     bar_256(1);
     r = t & 15;
     const int k = t >> 4;
@@ -179,7 +199,8 @@ struct ClusterChol {
   __device__ __forceinline__ double* block(int I, int K) const { return m.blk + ((int64_t)cl_slot(plan[I]) + K) * 256; }
   __device__ __forceinline__ bool own(int I) const { return cl_rank(plan[I]) == rank; }
   __device__ __forceinline__ void keep_inverse(int p) {
-    if (own(p) && threadIdx.x < 256) block(p, p)[threadIdx.x] = m.ybuf[(p & 1) * 256 + threadIdx.x];
+    if (own(p) && threadIdx.x < 256 && m.has(block(p, p) + threadIdx.x))
+      block(p, p)[threadIdx.x] = m.ybuf[(p & 1) * 256 + threadIdx.x];
   }
 
   // Own rows' L blocks of panel p, in place and into every rank's panel buffer.
@@ -192,10 +213,13 @@ struct ClusterChol {
       int r, c;
       double* at = block(I, p);
       const double l = panel_entry(at, m.ybuf + (p & 1) * 256, t, r, c);
+      double* pb = m.pbuf + I * 256 + c * 16 + r;
+      if (m.has(pb)) {
 #pragma unroll 4
-      for (int q = rank0_rows ? 0 : 1; q < size; ++q) cl_map(m.pbuf, q)[I * 256 + c * 16 + r] = l;
+        for (int q = rank0_rows ? 0 : 1; q < size; ++q) *cl_map(pb, q) = l;
+      }
       bar_256(2 + half);  // the half's threads have read the block
-      at[c * 16 + r] = l;
+      if (m.has(at + c * 16 + r)) at[c * 16 + r] = l;
     }
   }
 
@@ -208,7 +232,6 @@ struct ClusterChol {
     int total = 0;
     for (int x = x0; x < nrows; ++x) total += rows[x] - p;
     double* next = rank == 0 ? m.cbuf : cl_map(m.cbuf, 0);
-    next += ((p + 1) & 1) * 512;
     for (int u = threadIdx.x; u < total * 64; u += kClThreads) {
       int b = u >> 6, x = x0;
       while (b >= rows[x] - p) b -= rows[x++] - p;
@@ -233,12 +256,17 @@ struct ClusterChol {
       e0.y -= acc[1][0];
       e1.x -= acc[0][1];
       e1.y -= acc[1][1];
-      *reinterpret_cast<double2*>(o) = e0;
-      *reinterpret_cast<double2*>(o + 16) = e1;
+      if (m.has(reinterpret_cast<double2*>(o + 16))) {
+        *reinterpret_cast<double2*>(o) = e0;
+        *reinterpret_cast<double2*>(o + 16) = e1;
+      }
       if (I == p + 2) {
-        double* w = next + (K - (p + 1)) * 256 + k0 * 16 + r0;
-        *reinterpret_cast<double2*>(w) = e0;
-        *reinterpret_cast<double2*>(w + 16) = e1;
+        const int at = ((p + 1) & 1) * 512 + (K - (p + 1)) * 256 + k0 * 16 + r0;
+        double* w = next + at;
+        if (m.has(reinterpret_cast<double2*>(m.cbuf + at + 16))) {
+          *reinterpret_cast<double2*>(w) = e0;
+          *reinterpret_cast<double2*>(w + 16) = e1;
+        }
       }
     }
   }
@@ -266,11 +294,11 @@ struct ClusterChol {
         for (int q = 0; q < 4; ++q) {
           const int u = u0 + q * kClThreads, r = u / per, c = u - r * per, i = I * CNB + r;
           if (r >= CNB) break;
-          if (i < n && c <= i) {
+          if (i < n && c <= i && GNM_IN((int64_t)i * n + c, (int64_t)n * n)) {
             H[(int64_t)i * n + c] = h[q];
             H[(int64_t)c * n + i] = h[q];
           }
-          row[c * 16 + r] = h[q];
+          if (m.has(row + c * 16 + r)) row[c * 16 + r] = h[q];
         }
       }
     }
@@ -280,7 +308,7 @@ struct ClusterChol {
       if (t < 256 && r >= k && r < n) v = entry(r, k);
       for (int u = t; u < 512; u += kClThreads) {  // blocks (1, 0) and (1, 1)
         const int i = CNB + (u & 15), c = ((u >> 8) * CNB) + ((u >> 4) & 15);
-        m.cbuf[u] = (i < n && c <= i) ? entry(i, c) : 0.0;
+        if (m.has(m.cbuf + u)) m.cbuf[u] = (i < n && c <= i) ? entry(i, c) : 0.0;
       }
     }
     cl_arrive();
@@ -339,7 +367,7 @@ struct ClusterChol {
       const int p0 = p * CNB, nb = min(CNB, n - p0);
       if (I == p) {
         const double z = dot(block(p, p) + r * CNB, 1, v.b + p0, nb);
-        if (r < nb)
+        if (r < nb && m.has(v.z + i))
 #pragma unroll 4
           for (int q = 0; q < size; ++q) cl_map(v.z, q)[i] = z;
       }
@@ -347,11 +375,11 @@ struct ClusterChol {
       cl_wait();
       if (I > p) {
         const double s = dot(block(I, p) + r, 16, v.z + p0, nb);
-        if (live) v.b[i] -= s;
+        if (live && m.has(v.b + i)) v.b[i] -= s;
         __syncwarp(hm);
       }
     }
-    if (live) v.b[i] = v.z[i];
+    if (live && m.has(v.b + i)) v.b[i] = v.z[i];
     __syncwarp();
     for (int p = nblk - 1; p >= 0; --p) {
       const int p0 = p * CNB, nb = min(CNB, n - p0);
@@ -359,19 +387,20 @@ struct ClusterChol {
       if (own(p)) {  // uniform over the CTA
         if (I == p) {
           const double z = dot(block(p, p) + r, CNB, v.b + p0, nb);
-          if (r < nb)
+          if (r < nb && m.has(out + i))
 #pragma unroll 4
             for (int q = 0; q < size; ++q) cl_map(out, q)[i] = z;
         }
         __syncthreads();
         for (int j = threadIdx.x; j < p0; j += kClThreads) {
-          cl_map(s, cl_rank(plan[j >> 4]))[j] = dot(block(p, j >> 4) + (j & 15) * 16, 1, out + p0, nb);
+          const double d = dot(block(p, j >> 4) + (j & 15) * 16, 1, out + p0, nb);
+          if (m.has(s + j)) cl_map(s, cl_rank(plan[j >> 4]))[j] = d;
         }
       }
       cl_arrive();
       cl_wait();
       if (I >= 0 && I < p) {
-        v.b[i] -= s[i];
+        if (m.has(v.b + i)) v.b[i] -= s[i];
         __syncwarp(hm);
       }
     }
@@ -396,7 +425,7 @@ struct ClusterChol {
 #pragma unroll
       for (int q = 0; q < 16; ++q) cur[q] = nxt[q];
     }
-    v.b[i] = v.rhs[i] - acc;
+    if (m.has(v.b + i)) v.b[i] = v.rhs[i] - acc;
   }
 
   // S y for this thread's row (srow_dot's order), the row block's rows of S
@@ -431,7 +460,7 @@ struct ClusterChol {
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
           const int row = 2 * q + (lane >> 4);
-          tile[row * 16 + (r ^ row)] = cur[q];
+          if (m.has(tile + row * 16 + (r ^ row))) tile[row * 16 + (r ^ row)] = cur[q];
         }
         fetch(c0 + 16);  // zeros past the last column
         __syncwarp();

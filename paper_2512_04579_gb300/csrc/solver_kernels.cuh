@@ -615,7 +615,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_solve_cluster(SolveArgs a) {
   const int n = I.n, tid = threadIdx.x;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int fail[2], nrows;
-  __shared__ int rows[kClMaxBlocks];
+  __shared__ int rows[kClMaxRows];
   __shared__ double red[32];
   ClusterChol cc;
   cc.size = cl_size();
@@ -632,10 +632,11 @@ __global__ void __launch_bounds__(kClThreads, 1) k_solve_cluster(SolveArgs a) {
   cc.m.col = v + 1792;
   cc.m.pbuf = v + 1860;
   cc.m.blk = cc.m.pbuf + (int64_t)cc.nblk * 256;
+  cc.m.words = cl_dyn_words();
   if (tid == 0) {
     int c = 0;
     for (int q = 0; q < cc.nblk; ++q)
-      if (cl_rank(cc.plan[q]) == cc.rank) rows[c++] = q;
+      if (cl_rank(cc.plan[q]) == cc.rank && GNM_IN(c, kClMaxRows)) rows[c++] = q;
     nrows = c;
   }
   bool r0 = false;
@@ -677,8 +678,8 @@ __global__ void __launch_bounds__(kClThreads, 1) k_solve_cluster(SolveArgs a) {
   double gsq = 0.0;
   for (int j = tid; j < n; j += blockDim.x) {
     const double gj = a.g[I.o_U + j];
-    w.rhs[j] = -gj;
-    w.b[j] = -gj;
+    if (cc.m.has(w.rhs + j)) w.rhs[j] = -gj;
+    if (cc.m.has(w.b + j)) w.b[j] = -gj;
     gsq += gj * gj;
   }
   if (cc.rank == 0) {
@@ -701,13 +702,14 @@ __global__ void __launch_bounds__(kClThreads, 1) k_solve_cluster(SolveArgs a) {
     cc.residual(w, H);
     __syncwarp();
     cc.substitute(w, w.dx);
-    for (int j = tid; j < n; j += blockDim.x) w.x[j] += w.dx[j];
+    for (int j = tid; j < n; j += blockDim.x)
+      if (cc.m.has(w.x + j)) w.x[j] += w.dx[j];
     __syncthreads();
   }
   for (int j = tid; j < n; j += blockDim.x) {
     const float h = (float)w.x[j];
-    w.yh[j] = h;
-    w.yl[j] = (float)(w.x[j] - (double)h);
+    if (cc.m.has(w.yh + j)) w.yh[j] = h;
+    if (cc.m.has(w.yl + j)) w.yl[j] = (float)(w.x[j] - (double)h);
   }
   __syncthreads();
   const TA* P = reinterpret_cast<const TA*>(a.P) + I.o_P;
@@ -720,7 +722,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_solve_cluster(SolveArgs a) {
       a.delta[I.o_U + i] = acc;
       a.y[I.o_U + i] = w.x[i];
     }
-    cl_map(w.delta, 0)[i] = acc;
+    if (cc.m.has(w.delta + i)) cl_map(w.delta, 0)[i] = acc;
   }
   cl_arrive();
   cl_wait();
