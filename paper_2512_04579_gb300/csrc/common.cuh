@@ -387,14 +387,21 @@ struct Chain {
   }
 };
 
-// 1 / sqrt(q) of a link's squared length.  FAST is the hardware approximation
-// alone; rsqrtf adds three instructions per link that rescale a subnormal q, and
-// is bitwise the same for every other q.  For a subnormal q (a link shorter
-// than 1.1e-19) FAST gives infinity, which no later step takes back: it makes
-// the rollout's cost infinite or NaN.  So the sample kernels roll out with FAST
-// and run the rare warp that ends with a non-finite cost again without it
-// (samples phase of 256 chains, M = 10, N = 100, K = 2048: 2.01 -> 1.85 ms; 16 of
-// M = 32, N = 200, K = 4096: 2.32 -> 2.16; 64 of M = 16: 1.01 -> 0.92).
+// 1 / sqrt(q) of a link's squared length.  FAST is rsqrt.approx.ftz, which
+// flushes a subnormal q to zero; for every other q it gives rsqrtf's bits
+// (tests/test_link_rsqrt_all_gpu.py goes through them all).  For a subnormal q (a
+// link shorter than 1.1e-19) it gives infinity, which no later step takes back:
+// the rollout's cost becomes infinite or NaN.  So the sample kernels roll out with
+// FAST and run a warp that ends with a non-finite cost again without it (samples
+// phase of 256 chains, M = 10, N = 100, K = 2048: 2.01 -> 1.85 ms; 16 of M = 32, N =
+// 200, K = 4096: 2.32 -> 2.16; 64 of M = 16: 1.01 -> 0.92).
+// What it costs: a diverged rollout ends the same way, so a warp with a dropped
+// sample takes up to twice the time.  The 256 chains with scales at which 1.7 % of
+// the pairs diverge: 1.94 ms without FAST, 2.93 with it; 48 % (and half the
+// instances fail and are skipped): 1.20 and 2.32.  Telling the two apart cost
+// batches without drops more than it saved: the smallest q kept per link 1.91 ms
+// (64 chains of M = 13: 425 -> 474 us), the step repeated in place 1.90 (M = 64: 2.94
+// -> 4.11 ms), the dropped pairs alone run again 1.87 (M = 9: 270 -> 294 us).
 template <bool FAST>
 __device__ __forceinline__ float link_rsqrt(float q) {
   if constexpr (!FAST) return rsqrtf(q);
