@@ -51,7 +51,7 @@ unsigned int check_count_mlp();
 // Threads of a thread-per-rollout sample CTA: an antithetic pair takes two, a
 // one-sided sample one.  FP64 rollouts are bound by each SM sub-partition's FP64
 // issue, so smaller CTAs spread a small batch over more of them (one pendulum's
-// samples 254 -> 234 us); FP32 ones are faster with 128 (256 chains of M = 10: 1.85
+// samples 259 -> 238 us); FP32 ones are faster with 128 (256 chains of M = 10: 1.85
 // ms, 2.01 with 64).
 constexpr int sample_threads(bool fp64) { return fp64 ? 64 : 128; }
 constexpr int kPadK = 64;            // sample-dimension padding of dR / W rows

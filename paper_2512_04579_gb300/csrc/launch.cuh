@@ -73,7 +73,7 @@ void fill(Launchers* o) {
 // 1 / 4 / 8 / 16 lanes per candidate, M = 16 0.152 / 0.094 / 0.107 ms with 4 / 8 / 16.
 // Two warps per CTA: a candidate's rollout is one serial chain, so a batch's
 // few warps belong on as many SM sub-partitions as there are (256-thread CTAs
-// put eight on one SM: 16 chains of M = 32 258 us, 138 now; eight FP64 chains
+// put eight on one SM: 16 chains of M = 32 258 us, 125 now; eight FP64 chains
 // of M = 10 2.10 ms, 1.08 now; 256 chains of M = 10 84, 82 us).
 template <typename T, int FL, int G, int FX = 0>
 void launch_line_group(const RollArgs& a, int ncand_total, cudaStream_t s) {

@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(kContractThreads<MT>, 3 - MT) k_contract_tc(co
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const uint32_t done = su32(bars + 3 * STAGES);
-  // stage layout: A sub-tile 0, [A sub-tile 1,] B rows 0-127, B rows 128-255 (8 KB each)
+  // stage layout: A sub-tile 0, [A sub-tile 1,] B rows 0-127, B rows 128-255 (16 KB each)
 
   if (warp == 0 && lane == 0) {
     // ---------------- TMA producer
@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(kGramThreads, BF ? 2 : 1) k_gram_tc(const CUte
   const TcJob J = jobs[tl.x];
   const int mt = tl.w & 3;
   const bool diag = (tl.w & 4) != 0;
-  const int q0 = (tl.w >> 3) & 1;  // BF16: the diagonal tile's second sub-tile alone
+  const int q0 = (tl.w >> 3) & 1;  // one-sub-tile tiles: the diagonal tile's second sub-tile alone
   const int row_org = tl.y, col_org = tl.z;
   const int kept = min(BN, J.Nc - col_org);  // output columns of this tile = B rows
   const int kept_b = diag ? min(kept, BM * (q0 + mt)) : kept;  // B rows the MMAs read
@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(kGramThreads, BF ? 2 : 1) k_gram_tc(const CUte
   // BF16: 256 B rows [, 128 A rows], each split in place
   const int RING = BF ? ring : RING_BYTES;
   const int stage_bytes = BF ? (diag ? nbox * BM * RB : (BN + BM) * RB) : (diag ? 2 * B_BYTES : 2 * (B_BYTES + A_BYTES));
-  const int stages = min(MAXST, RING / stage_bytes);  // TF32: 3 (diagonal) or 2; BF16: 6, 3 or 2
+  const int stages = min(MAXST, RING / stage_bytes);  // TF32: 3 (diagonal) or 2; BF16: 6, 3 or 2 (192 KB ring: 12, 6 or 4)
   const int a_off = BF ? BN * RB : 2 * B_BYTES;              // A rows of an off-diagonal stage
   const uint32_t tx_bytes = (uint32_t)(nbox * BM * RB + (diag ? 0 : BM * RB));
   const uint32_t tcols = mt == 2 ? 2 * TMEM_COLS : TMEM_COLS;
@@ -834,7 +834,7 @@ gnmppi_status tc_plan_create(const std::vector<InstDesc>& desc, void* dRW, const
     jg.out_off = d.o_nn;
     jg.ldc = d.n;
     jg.ccut = d.n;
-    // nR beyond kGramChunkCols: one job per column chunk into the FP64 chunk
+    // nR beyond kGramChunkCols: one job per column chunk into the FP32 chunk
     // buffer, added up by k_gram_reduce
     const int gchunk = kGramChunkCols / KBLK;
     const int nchunks = (jg.nkb + gchunk - 1) / gchunk;
